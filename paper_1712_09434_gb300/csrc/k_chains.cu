@@ -14,8 +14,8 @@ namespace tpc {
 namespace {
 
 // Kept up-link of every cluster (-1 if none or not mutual), and the successors 2 and 4 links
-// further: a chain walk then takes four links per dependent load.  The arrays live in the
-// selection's claim and owner words, which the selection re-initialises before use.
+// further: a chain walk then takes four links per dependent load.  The first two live in the
+// selection's claim words, which the selection re-initialises before use.
 struct Jumps {
     int32_t *n1, *n2, *n4;
 };
@@ -23,7 +23,7 @@ __device__ __forceinline__ Jumps jumps_of(const Work &W) {
     Jumps j;
     j.n1 = reinterpret_cast<int32_t *>(W.claim);
     j.n2 = reinterpret_cast<int32_t *>(W.claim) + (W.n_clusters + 1);
-    j.n4 = reinterpret_cast<int32_t *>(W.owner);
+    j.n4 = W.jump4;
     return j;
 }
 
@@ -123,7 +123,7 @@ void launch_chains(const Work &W, cudaStream_t s) {
     k_mutual<<<gj, 256, 0, s>>>(W);
     int32_t *n1 = reinterpret_cast<int32_t *>(W.claim), *n2 = n1 + (W.n_clusters + 1);
     k_jump<<<gj, 256, 0, s>>>(W, n1, n2);
-    k_jump<<<gj, 256, 0, s>>>(W, n2, reinterpret_cast<int32_t *>(W.owner));
+    k_jump<<<gj, 256, 0, s>>>(W, n2, W.jump4);
     k_chain_count<<<grid, block, 0, s>>>(W);
     scan_exclusive(W.bin_cnt, W.chain_off, W.nbins, nullptr, W.counters + CNT_NCHAINS, W.scan_tmp,
                    W.scan_tmp_len, s);

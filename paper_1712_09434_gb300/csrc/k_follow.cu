@@ -286,8 +286,7 @@ __global__ void __launch_bounds__(128) k_follow(Work W, const int32_t *perm) {
 void launch_follow(const Work &W, cudaStream_t s) {
     const int block = W.tune.block[3] > 0 ? W.tune.block[3] : 128;
     const int grid = W.tune.grid[3] > 0 ? W.tune.grid[3] : W.sm_count * 8;
-    // the permutation lives in the selection states, which the selection writes before it reads
-    int32_t *perm = W.cstate;
+    int32_t *perm = W.perm;
     k_follow_order<<<W.sm_count * 8, 256, 0, s>>>(W, perm);
     if (W.rules & TPC_RULE_SKIP_ROW)
         k_follow<true><<<grid, block, 0, s>>>(W, perm);

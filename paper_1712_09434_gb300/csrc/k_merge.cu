@@ -14,19 +14,39 @@ namespace tpc {
 
 namespace {
 
-__device__ __forceinline__ uint32_t key_of(int n_rows, int n_hits, int local) {
-    return ((uint32_t)(n_rows - n_hits) << 23) | (uint32_t)local;
-}
-
 __device__ __forceinline__ int n_chains_of(const Work &W) {
     const int n = W.counters[CNT_NCHAINS];
     return n < W.cap_chains ? n : W.cap_chains;
 }
 
-// first candidate index of the (event, sector) of candidate t
-__device__ __forceinline__ int sector_base(const Work &W, int t) {
-    const int bin = W.chain_bin[t];
-    return W.chain_off[bin - bin % W.nr];
+// Kept hits of an accepted candidate: a bit per row of its row range [r0, r1], from r0 on.
+struct Kept {
+    const uint32_t *w;
+    int r0, r1;
+    __device__ __forceinline__ bool has(int r) const { return (w[(r - r0) >> 5] >> ((r - r0) & 31)) & 1u; }
+    // row of the first kept hit
+    __device__ __forceinline__ int first() const {
+        for (int j = 0; j <= (r1 - r0) >> 5; j++)
+            if (w[j]) return r0 + 32 * j + __ffs(w[j]) - 1;
+        return -1;
+    }
+    // row of the last kept hit and of the kept hit `back` positions before it (-1 if there is none)
+    __device__ __forceinline__ void last(int back, int &rl, int &rb) const {
+        rl = rb = -1;
+        for (int j = (r1 - r0) >> 5; j >= 0; j--) {
+            uint32_t m = w[j];
+            while (m) {
+                const int bit = 31 - __clz(m), r = r0 + 32 * j + bit;
+                if (rl < 0) rl = r;
+                if (back-- == 0) { rb = r; return; }
+                m &= ~(1u << bit);
+            }
+        }
+    }
+};
+__device__ __forceinline__ Kept kept_of(const Work &W, int t) {
+    const int rr = W.cand_rows[t];
+    return Kept{W.kept + (size_t)t * kept_words(W.nr), rr & 0xffff, rr >> 16};
 }
 
 // ends of accepted segments; reset of the merge arrays
@@ -39,23 +59,14 @@ __global__ void k_merge_ends(Work W) {
         W.next[t] = -1;
         W.prev[t] = -1;
         if (W.seg_n[t] < N_MIN) continue;
-        const uint32_t key = key_of(W.nr, W.cand_n[t], t - sector_base(W, t));
-        const int rr = W.cand_rows[t];
+        const Kept kept = kept_of(W, t);
         const int32_t *sl = W.cand_slots + (size_t)t * W.nr;
-        int ring_h[MERGE_BACK + 1], ring_r[MERGE_BACK + 1];
-        int first = -1, rf = 0, cnt = 0;
-        for (int r = rr & 0xffff; r <= (rr >> 16); r++) {
-            const int h = sl[r];
-            if (h < 0 || W.owner[h] != key) continue;
-            if (first < 0) { first = h; rf = r; }
-            ring_h[cnt % (MERGE_BACK + 1)] = h;
-            ring_r[cnt % (MERGE_BACK + 1)] = r;
-            cnt++;
-        }
-        if (cnt <= MERGE_BACK) { set_status(W, ST_BOUNDS); continue; }
+        const int rf = kept.first();
+        int rL, rB;
+        kept.last(MERGE_BACK, rL, rB);
+        if (rB < 0) { set_status(W, ST_BOUNDS); continue; }
+        const int first = sl[rf], hL = sl[rL], hB = sl[rB];
         const int sector = (W.chain_bin[t] % (W.ns * W.nr)) / W.nr;
-        const int iL = (cnt - 1) % (MERGE_BACK + 1), iB = (cnt - 1 - MERGE_BACK) % (MERGE_BACK + 1);
-        const int hL = ring_h[iL], rL = ring_r[iL], hB = ring_h[iB], rB = ring_r[iB];
         W.inend[t] = make_int4(g.xtab[rf], W.pad[first], W.tim[first], sector);
         atomicMax(W.sec_ymax + W.chain_bin[t] / (W.ns * W.nr) * W.ns + sector, abs((int)W.pad[first]));
         atomicAdd(W.bin_cnt + (W.chain_bin[t] - W.chain_bin[t] % W.nr) + rf, 1);
@@ -118,14 +129,13 @@ __global__ void k_gap_back(Work W) {
         W.gap_bestT[t] = ~0ull;
         W.gap_bestS[t] = ~0ull;
         if (W.seg_n[t] < N_MIN) continue;
-        const uint32_t key = key_of(W.nr, W.cand_n[t], t - sector_base(W, t));
-        const int rr = W.cand_rows[t];
+        const Kept kept = kept_of(W, t);
         const int32_t *sl = W.cand_slots + (size_t)t * W.nr;
         Abg fy{}, fz{};
         int k = 0, rprev = 0, h0 = -1;
-        for (int r = rr >> 16; r >= (rr & 0xffff); r--) {
+        for (int r = kept.r1; r >= kept.r0; r--) {
+            if (!kept.has(r)) continue;
             const int h = sl[r];
-            if (h < 0 || W.owner[h] != key) continue;
             if (k == 0) {
                 h0 = h;
             } else if (k == 1) {
@@ -156,14 +166,13 @@ __global__ void k_gap_match(Work W) {
     const int n = n_chains_of(W);
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         if (W.seg_n[s] < N_MIN) continue;
-        const uint32_t key = key_of(W.nr, W.cand_n[s], s - sector_base(W, s));
-        const int rr = W.cand_rows[s];
+        const Kept kept = kept_of(W, s);
         const int32_t *sl = W.cand_slots + (size_t)s * W.nr;
         Abg fy{}, fz{};
         int k = 0, rprev = 0, h0 = -1, hl = -1;
-        for (int r = rr & 0xffff; r <= (rr >> 16); r++) {
+        for (int r = kept.r0; r <= kept.r1; r++) {
+            if (!kept.has(r)) continue;
             const int h = sl[r];
-            if (h < 0 || W.owner[h] != key) continue;
             if (k == 0) {
                 h0 = h;
             } else {
@@ -361,8 +370,10 @@ __global__ void k_track_count(Work W) {
     }
 }
 
-// One warp per track: the lanes read 32 row slots of a segment at a time and write its kept hits
-// in row order (ballot prefix), then move to the next segment of the merge chain.
+// One warp per track: the lanes take the row slots of a segment 32 at a time, TW_ILP groups loaded
+// together, and write its kept hits in row order (prefix of the kept bits), then move to the next
+// segment of the merge chain.
+constexpr int TW_ILP = 5;
 __global__ void k_track_write(Work W) {
     const int nt = min(W.counters[CNT_NTRACKS], W.cap_tracks);
     const int lane = threadIdx.x & 31;
@@ -371,27 +382,38 @@ __global__ void k_track_write(Work W) {
         int pos = W.trk_off[tid];
         int x = W.trk_head[tid], k = 0;
         do {
-            const uint32_t key = key_of(W.nr, W.cand_n[x], x - sector_base(W, x));
-            const int rr = W.cand_rows[x];
+            const Kept kept = kept_of(W, x);
             const int32_t *sl = W.cand_slots + (size_t)x * W.nr;
             const int sector = (W.chain_bin[x] % (W.ns * W.nr)) / W.nr;
-            for (int r0 = rr & 0xffff; r0 <= (rr >> 16); r0 += 32) {
-                const int r = r0 + lane;
-                const int h = r <= (rr >> 16) ? sl[r] : -1;
-                const bool kept = h >= 0 && W.owner[h] == key;
-                const unsigned m = __ballot_sync(0xffffffffu, kept);
-                if (kept) {
-                    const int p = pos + __popc(m & ((1u << lane) - 1u));
-                    if (p < W.cap_hits) {
-                        W.trk_hits[p] = h;
-                        W.label[h] = tid;
-                        W.trk_pack[2 * p] = (int32_t)((uint32_t)(W.pad[h] & 0xffff) | ((uint32_t)W.tim[h] << 16));
-                        W.trk_pack[2 * p + 1] = sector | (r << 16);
-                    } else {
-                        set_status(W, ST_CAPACITY);
-                    }
+            const int nwords = ((kept.r1 - kept.r0) >> 5) + 1;
+            for (int j0 = 0; j0 < nwords; j0 += TW_ILP) {
+                int h[TW_ILP], yz[TW_ILP];
+                unsigned m[TW_ILP];
+#pragma unroll
+                for (int j = 0; j < TW_ILP; j++) {
+                    m[j] = j0 + j < nwords ? kept.w[j0 + j] : 0u;
+                    const int r = kept.r0 + 32 * (j0 + j) + lane;
+                    h[j] = r <= kept.r1 ? sl[r] : -1;
                 }
-                pos += __popc(m);
+#pragma unroll
+                for (int j = 0; j < TW_ILP; j++)
+                    if ((m[j] >> lane) & 1u)
+                        yz[j] = (int)((uint32_t)(W.pad[h[j]] & 0xffff) | ((uint32_t)W.tim[h[j]] << 16));
+#pragma unroll
+                for (int j = 0; j < TW_ILP; j++) {
+                    if ((m[j] >> lane) & 1u) {
+                        const int p = pos + __popc(m[j] & ((1u << lane) - 1u));
+                        const int r = kept.r0 + 32 * (j0 + j) + lane;
+                        if (p < W.cap_hits) {
+                            W.trk_hits[p] = h[j];
+                            W.label[h[j]] = tid;
+                            reinterpret_cast<int2 *>(W.trk_pack)[p] = make_int2(yz[j], sector | (r << 16));
+                        } else {
+                            set_status(W, ST_CAPACITY);
+                        }
+                    }
+                    pos += __popc(m[j]);
+                }
             }
             x = W.next[x];
             k++;

@@ -101,8 +101,9 @@ size_t layout(tpc_ctx *c, char *base) {
     carve(cur, w.cand_rows, C);
     carve(cur, w.cand_slots, C * c->hgeom.n_rows);
     carve(cur, w.claim, 2 * N);
-    carve(cur, w.owner, N);
-    carve(cur, w.cstate, C);
+    carve(cur, w.jump4, N);
+    carve(cur, w.perm, C);
+    carve(cur, w.kept, C * kept_words(c->hgeom.n_rows));
     carve(cur, w.seg_n, C);
     carve(cur, w.bestT, C);
     carve(cur, w.bestS, C);

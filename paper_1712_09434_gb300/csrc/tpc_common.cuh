@@ -92,18 +92,19 @@ struct Work {
     int32_t *up, *down;       // [N]
     // chains (S3, S4)
     int32_t *clen;            // [N] kept chain length at its start cluster, else 0
+    int32_t *jump4;           // [N] successor four links further
     int32_t *bin_cnt;         // [nbins + 1] chains starting in the bin
     int32_t *chain_off;       // [nbins + 1] exclusive scan of bin_cnt
     int32_t *chain_start, *chain_len, *chain_bin;   // [cap_chains]
     int cap_chains;
     // following (S5)
+    int32_t *perm;            // [cap_chains] order in which it takes the chains
     int32_t *cand_n;          // [cap_chains]
     int32_t *cand_rows;       // [cap_chains] row0 | row1 << 16
     int32_t *cand_slots;      // [cap_chains * n_rows] cluster per row inside [row0, row1], else -1
     // selection (S6)
-    uint32_t *claim;          // [2N] 64-bit round-tagged claims
-    uint32_t *owner;          // [N]  key of the accepted candidate owning the cluster
-    int32_t *cstate;          // [cap_chains] selection state
+    uint32_t *claim;          // [2N] 64-bit claims: (round, or ~0 once owned) << 32 | ~key
+    uint32_t *kept;           // [cap_chains * kept_words(n_rows)] bit per row from row0 on: the kept hits
     int32_t *seg_n;           // [cap_chains] kept hits, 0 if rejected
     // merge (S7)
     unsigned long long *bestT, *bestS;  // [cap_chains]
@@ -145,6 +146,9 @@ enum {
     CNT_BINS_BAD = 7,         // set when the caller's bin offsets fail the check
     CNT_Q0 = 8,               // work-queue heads, one per kernel
 };
+
+// words of the kept-hit mask of a candidate
+__host__ __device__ inline int kept_words(int n_rows) { return (n_rows + 31) / 32; }
 
 __host__ __device__ inline int pstart_of(int32_t off, int b) { return ((off + 7) & ~7) + 8 * b; }
 
