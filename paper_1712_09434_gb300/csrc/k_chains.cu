@@ -27,6 +27,9 @@ __device__ __forceinline__ Jumps jumps_of(const Work &W) {
     return j;
 }
 
+// last cluster of the chain that starts at c; in the packed track hits, which are written later
+__device__ __forceinline__ int32_t *chain_ends(const Work &W) { return W.trk_pack; }
+
 __global__ void k_mutual(Work W) {
     const Jumps J = jumps_of(W);
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < W.n_clusters; c += gridDim.x * blockDim.x) {
@@ -43,8 +46,9 @@ __global__ void k_jump(Work W, const int32_t *src, int32_t *dst) {
 }
 
 // chain length from a start cluster, or 0 if c is not a start (a start has a kept up-link and no
-// kept down-link); the count of clusters along the kept up-links, at most max_len
-__device__ int chain_length(const Work &W, const Jumps &J, int c, int max_len) {
+// kept down-link); the count of clusters along the kept up-links, at most max_len.  The last
+// cluster goes to *last.
+__device__ int chain_length(const Work &W, const Jumps &J, int c, int max_len, int *last) {
     if (J.n1[c] < 0) return 0;
     const int d = W.down[c];
     if (d >= 0 && J.n1[d] == c) return 0;
@@ -63,6 +67,7 @@ __device__ int chain_length(const Work &W, const Jumps &J, int c, int max_len) {
         x = y;
         len++;
     }
+    *last = x;
     return len;
 }
 
@@ -75,9 +80,11 @@ __global__ void __launch_bounds__(256) k_chain_count(Work W) {
         const int c0 = W.bin_off[b], c1 = W.bin_off[b + 1];
         int cnt = 0;
         for (int c = c0 + lane; c < c1; c += 32) {
-            int len = chain_length(W, J, c, max_len);
+            int last;
+            int len = chain_length(W, J, c, max_len, &last);
             if (len < N_SEED) len = 0;
             W.clen[c] = len;
+            if (len > 0) chain_ends(W)[c] = last;
             cnt += len > 0;
         }
 #pragma unroll
@@ -100,8 +107,11 @@ __global__ void __launch_bounds__(256) k_chain_write(Work W) {
                 const int p = pos + __popc(m & ((1u << lane) - 1u));
                 if (p < W.cap_chains) {
                     W.chain_start[p] = c;
+                    W.chain_last[p] = chain_ends(W)[c];
                     W.chain_len[p] = len;
                     W.chain_bin[p] = b;
+                    W.cand_n[p] = len;      // the following adds what it finds and the row range
+                    W.cand_rows[p] = 0;
                 } else {
                     set_status(W, ST_CAPACITY);
                 }

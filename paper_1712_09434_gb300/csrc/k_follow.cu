@@ -4,106 +4,139 @@
 // shifts, int64) so that the hit lists are bit-identical to an independent FP64 implementation;
 // the floating-point Kalman filter is used for the parameters only (S8).
 //
-// The filter runs along the whole chain, then extends it row by row outwards, then (re-initialised
-// from the other end) inwards: predict, look up the nearest cluster (minimum (d^2, index)) within a
+// A chain is followed by two threads at once: one filters along it in ascending rows and extends it
+// row by row outwards, the other filters in descending rows and extends it inwards.  A step: predict, look up the nearest cluster (minimum (d^2, index)) within a
 // radius that grows with consecutive misses in the row's Z-slab grid, update.  A candidate is
 // stored as one cluster per row (-1 for a miss) between its first and last row.  The chains are
 // taken in an order that groups chains of equal length and nearby start rows in a warp (below).
+//
+// What bounds it: the dependent loads of one thread's steps (link, coordinates; slab offsets, search)
+// and the instructions of a divergent search, over the threads in flight.  Two threads a chain halve
+// the serial length, the filter runs in 32-bit words where the geometry allows it, which also leaves
+// registers for ten blocks of 128 threads a multiprocessor, and the row offset and the found
+// cluster's index are off the step's critical path.  Measured (one thread a chain with a 64-bit
+// filter -> this): 64 events of 1.14 M chains 4.15 -> 3.02 ms, a central event 861 -> 643 us, a
+// 5,000-track event 446 -> 360 us, one sector of 138 chains 350 -> 190 us; with the 64-bit filter
+// 3.79 ms, 746, 331 and 213 us.  Reading a slab four entries at a time instead of by binary search
+// was slower where rows are dense (4.0 ms, 802 us).
 #include "tpc_common.cuh"
 
 namespace tpc {
 
 namespace {
 
+// The filter word T is int64, or int32 for geometries with ymax <= 16383 and zmax <= 32767 (narrow):
+// then a Q16 coordinate fits 32 bits, with Z shifted by -16384 so that one step never carries a
+// prediction past the word (a step moves less than 16384 LSB: the velocity that a track can build
+// up inside the drift range at 343 LSB per residual stays below that).  Sums and differences are
+// exact modulo 2^32 in any case, so only the reading of a prediction could be wrong, for a hit more
+// than 16384 LSB beyond the drift range; such a chain is not extended (it would stop at once).
+template <class T>
 struct Abg {
-    long long p, v, a;
+    static constexpr int ZB = sizeof(T) == 4 ? 16384 : 0;   // Z as the filter holds it: z - ZB
+    T p, v, a;
 };
+template <class T>
+__device__ __forceinline__ T q16(int m) {
+    if constexpr (sizeof(T) == 4) return (T)((uint32_t)m << 16);
+    else return (T)m * 65536;
+}
 
 // state at m0 with the velocity of the step to m1, drow = 1 or 2 rows further (2 across a row that
 // a link skips; the division is exact)
-__device__ __forceinline__ void abg_init(Abg &f, long long m0, long long m1, int drow) {
-    f.p = m0 * 65536;
-    f.v = (m1 - m0) * (65536 / drow);
+template <class T>
+__device__ __forceinline__ void abg_init(Abg<T> &f, int m0, int m1, int drow) {
+    f.p = q16<T>(m0);
+    f.v = (T)(m1 - m0) * (65536 / drow);
     f.a = 0;
 }
-__device__ __forceinline__ void abg_predict(Abg &f) {
+template <class T>
+__device__ __forceinline__ void abg_predict(Abg<T> &f) {
     f.p += f.v + (f.a >> 1);
     f.v += f.a;
 }
-__device__ __forceinline__ void abg_update(Abg &f, long long m) {
-    const long long e = m * 65536 - f.p;
+template <class T>
+__device__ __forceinline__ void abg_update(Abg<T> &f, int m) {
+    const T e = q16<T>(m) - f.p;
     f.p += e >> 1;
     f.v += e >> 3;
     f.a += e >> 5;
 }
-__device__ __forceinline__ int q16_round(long long p) { return (int)((p + 32768) >> 16); }
+template <class T>
+__device__ __forceinline__ int q16_round(T p) { return (int)((p + 32768) >> 16); }
+constexpr int NARROW_YMAX = 16383, NARROW_ZMAX = 32767, NARROW_ZHIT = 49151;
 __device__ __forceinline__ int slab_of(int z) { int s = z >> ZB_SHIFT; return s < NZB - 1 ? s : NZB - 1; }
 
-__device__ __forceinline__ int lower_y(const int32_t *yz, int lo, int hi, int y) {
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if ((int)(int16_t)(__ldg(yz + mid) & 0xffff) < y) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
-// Nearest cluster of a row bin to (py, pz) with d^2 <= w^2: row-local index, or -1; its packed
-// (Y, Z) goes to *yz (the grid payload, so the cluster arrays need not be read again).
-__device__ int nearest(const Work &W, int bin, int py, int pz, int w, int32_t *yz_out) {
-    const int c0 = __ldg(W.bin_off + bin);
-    const int32_t *yz = W.gyz + pstart_of(c0, bin);
-    const uint16_t *loc = W.gloc + pstart_of(c0, bin);
-    const uint16_t *zo = W.zoff + (size_t)bin * ZOFF_STRIDE;
+// Nearest cluster of a row (its grid entries yz, indices loc, slab offsets zo) to (py, pz) with
+// d^2 <= w^2 (w < 512): its position in the row's grid, or -1; its packed (Y, Z) goes to *yz_out
+// (the cluster arrays need not be read again).  Of equal distances the smallest index counts.
+__device__ __forceinline__ int nearest(const int32_t *yz, const uint16_t *loc, const uint16_t *zo, int py, int pz,
+                                       int w, int32_t *yz_out) {
     const int zl = slab_of(max(pz - w, 0)), zh = slab_of(pz + w);
-    const long long w2 = (long long)w * w;
-    long long bd = w2 + 1;
-    int bl = 0x7fffffff;
+    const int w2 = w * w;
+    int bd = w2 + 1, bi = -1;
     int32_t bv = 0;
     for (int s = zl; s <= zh; s++) {
-        const int hi = __ldg(zo + s + 1);
-        for (int i = lower_y(yz, __ldg(zo + s), hi, py - w); i < hi; i++) {
+        int a = __ldg(zo + s), e = __ldg(zo + s + 1);
+        const int hi = e;
+        while (a < e) {
+            const int mid = (a + e) >> 1;
+            if ((int)(int16_t)(__ldg(yz + mid) & 0xffff) < py - w) a = mid + 1; else e = mid;
+        }
+        for (int i = a; i < hi; i++) {
             const int32_t v = __ldg(yz + i);
-            const int y = (int16_t)(v & 0xffff);
-            if (y > py + w) break;
-            const long long dy = y - py, dz = (int)((uint32_t)v >> 16) - pz;
-            const long long d2 = dy * dy + dz * dz;
-            if (d2 > w2) continue;
-            const int l = __ldg(loc + i);
-            if (d2 < bd || (d2 == bd && l < bl)) { bd = d2; bl = l; bv = v; }
+            const int dy = (int)(int16_t)(v & 0xffff) - py;
+            if (dy > w) break;
+            const int dz = (int)((uint32_t)v >> 16) - pz;
+            if (abs(dz) > w) continue;
+            const int d2 = dy * dy + dz * dz;
+            if (d2 < bd || (d2 == bd && d2 <= w2 && __ldg(loc + i) < __ldg(loc + bi))) { bd = d2; bi = i; bv = v; }
         }
     }
     *yz_out = bv;
-    return bl == 0x7fffffff ? -1 : bl;
+    return bi;
 }
 
 // Extend from the filter state (already at row `row_last`) in direction dir; writes slots.
-// Returns the number of clusters found and the row of the last one in *row_end.
-__device__ int extend(const Work &W, const DevGeom &g, Abg &fy, Abg &fz, int rowbase_bin, int row_last, int dir,
-                      int32_t *slots, int *row_end) {
+// Returns the number of clusters found and the row of the last one in *row_end.  The next row's
+// cluster offset is loaded during a row, and a found cluster's index is stored during the next one.
+template <class T>
+__device__ __forceinline__ int extend(const Work &W, const DevGeom &g, Abg<T> &fy, Abg<T> &fz, int rowbase_bin,
+                                      int row_last, int dir, int nr, int32_t *slots, int *row_end) {
     int n = 0, misses = 0;
     *row_end = row_last;
-    for (int row = row_last + dir; row >= 0 && row < g.n_rows; row += dir) {
+    int row = row_last + dir;
+    int c_next = 0, pend = -1, pend_row = -1;      // a found cluster not stored yet
+    if (row >= 0 && row < nr) c_next = __ldg(W.bin_off + rowbase_bin + row);
+    while (row >= 0 && row < nr) {
+        const int c0 = c_next;
         abg_predict(fy);
         abg_predict(fz);
-        const int py = q16_round(fy.p), pz = q16_round(fz.p);
-        const long long av = fy.v < 0 ? -fy.v : fy.v;
-        if (abs(py) > g.ymax[row] || pz < 0 || pz > g.zmax || av > (long long)V_MAX * 65536) break;
+        const int py = q16_round(fy.p), pz = q16_round(fz.p) + Abg<T>::ZB;
+        if (abs(py) > g.ymax[row] || pz < 0 || pz > g.zmax || fy.v > (T)V_MAX * 65536 || fy.v < -(T)V_MAX * 65536) break;
         const int w = W_F0 + W_F1 * misses;
+        const int bin = rowbase_bin + row;
+        if (row + dir >= 0) c_next = __ldg(W.bin_off + bin + dir);
+        const int ps = pstart_of(c0, bin);
         int32_t v;
-        const int l = nearest(W, rowbase_bin + row, py, pz, w, &v);
-        if (l >= 0) {
-            const int h = __ldg(W.bin_off + rowbase_bin + row) + l;
+        const int i = nearest(W.gyz + ps, W.gloc + ps, W.zoff + (size_t)bin * ZOFF_STRIDE, py, pz, w, &v);
+        if (pend_row >= 0) slots[pend_row] = pend;
+        if (i >= 0) {
+            pend = c0 + (int)__ldg(W.gloc + ps + i);
+            pend_row = row;
             abg_update(fy, (int16_t)(v & 0xffff));
-            abg_update(fz, (int)((uint32_t)v >> 16));
-            slots[row] = h;
+            abg_update(fz, (int)((uint32_t)v >> 16) - Abg<T>::ZB);
             *row_end = row;
             n++;
             misses = 0;
         } else {
+            pend_row = -1;
             slots[row] = -1;
             if (++misses >= M_MISS) break;
         }
+        row += dir;
     }
+    if (pend_row >= 0) slots[pend_row] = pend;
     return n;
 }
 
@@ -154,144 +187,121 @@ __global__ void __launch_bounds__(256) k_follow_order(Work W, int32_t *perm) {
     }
 }
 
-// Each warp takes 32 x chunk chains at a time from the queue (no CTA barrier: a warp whose chains
-// end early takes the next ones while the others still follow theirs).  SKIP: chains may skip a
-// row (the skip-row rule); the plain instantiation keeps the plain reading's registers.
-template <bool SKIP>
-__global__ void __launch_bounds__(128) k_follow(Work W, const int32_t *perm) {
+// One step of the filter along the chain: `k` hits seen so far, the new one (y, z) `d` rows on.
+template <class T>
+struct ChainFilter {
+    Abg<T> fy, fz;
+    int m0y, m0z, k = 0;
+    __device__ __forceinline__ void hit(int y, int z0, int d) {
+        const int z = z0 - Abg<T>::ZB;
+        if (k == 0) {
+            m0y = y;
+            m0z = z;
+        } else {
+            if (k == 1) {   // state at the first hit with the velocity of the first step
+                abg_init(fy, m0y, y, d);
+                abg_init(fz, m0z, z, d);
+            }
+            for (int j = 0; j < d; j++) {
+                abg_predict(fy);
+                abg_predict(fz);
+            }
+            abg_update(fy, y);
+            abg_update(fz, z);
+        }
+        k++;
+    }
+};
+
+constexpr int FO_CTAS = 10;      // blocks a multiprocessor: 48 registers a thread
+
+// Each warp takes 32 x chunk tasks at a time from the queue (no CTA barrier: a warp whose chains
+// end early takes the next ones while the others still follow theirs).  Task groups of 32 come in
+// pairs: the outward tasks of 32 chains, then their inward tasks.  SKIP: chains may skip a row (the
+// skip-row rule); the plain instantiation keeps the plain reading's registers.
+template <bool SKIP, class T>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? FO_CTAS : 1) k_follow(Work W, const int32_t *perm) {
     const DevGeom &g = *W.geom;
     const int nr = g.n_rows;
     const int lane = threadIdx.x & 31;
     int n_chains = W.counters[CNT_NCHAINS];
     if (n_chains > W.cap_chains) n_chains = W.cap_chains;
-    const int chunk = 32 * (W.tune.chunk[3] > 0 ? W.tune.chunk[3] : 1);
+    const int n_groups = 2 * ((n_chains + 31) / 32);
+    const int chunk = W.tune.chunk[3] > 0 ? W.tune.chunk[3] : 1;
     int32_t *q = W.counters + CNT_Q0 + 3;
     for (;;) {
         int base = 0;
         if (lane == 0) base = atomicAdd(q, chunk);
         base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= n_chains) break;
-        for (int q = base + lane; q < base + chunk && q < n_chains; q += 32) {
-            const int t = perm[q];
-            const int start = W.chain_start[t], len = W.chain_len[t], bin = W.chain_bin[t];
+        if (base >= n_groups) break;
+        for (int gr = base; gr < base + chunk && gr < n_groups; gr++) {
+            const int i = (gr >> 1) * 32 + lane;
+            if (i >= n_chains) continue;
+            const int t = perm[i];
+            const bool out = (gr & 1) == 0;
+            const int len = W.chain_len[t], bin = W.chain_bin[t];
             const int row0 = bin % nr;
             const int rowbase = bin - row0;
             int32_t *slots = W.cand_slots + (size_t)t * nr;
-            Abg fy, fz;
-            int row_last;
-            if constexpr (!SKIP) {
-                // filter along the chain in ascending rows (consecutive rows), writing the chain hits
-                int x = start, m0y = 0, m0z = 0;
-                for (int k = 0; k < len; k++) {
-                    const int y = __ldg(W.pad + x), z = __ldg(W.tim + x);
-                    slots[row0 + k] = x;
-                    if (k == 0) {
-                        m0y = y;
-                        m0z = z;
-                    } else {
-                        if (k == 1) {   // state at the first hit with velocity m1 - m0
-                            abg_init(fy, m0y, y, 1);
-                            abg_init(fz, m0z, z, 1);
-                        }
-                        abg_predict(fy);
-                        abg_predict(fz);
-                        abg_update(fy, y);
-                        abg_update(fz, z);
-                    }
-                    if (k + 1 < len) x = W.up[x];
+            ChainFilter<T> f;
+            int z_last = 0;
+            const int dir = out ? 1 : -1;
+            int x = out ? W.chain_start[t] : W.chain_last[t];
+            const int32_t *link = out ? W.up : W.down;
+            int row = out ? row0 : row0 + len - 1;
+            if (SKIP && !out) {      // rows may be skipped: the last hit's row from its cluster
+                int hi = nr - 1;
+                while (row < hi) {
+                    const int mid = (row + hi + 1) >> 1;
+                    if (__ldg(W.bin_off + rowbase + mid) <= x) row = mid; else hi = mid - 1;
                 }
-                row_last = row0 + len - 1;
-            } else {
-                // the same with links that may skip a row: one filter step per pad row, a skipped
-                // row is a prediction without an update and a -1 slot
-                int x = start, m0y = 0, m0z = 0, row = row0, rprev = row0;
-                for (int k = 0; k < len; k++) {
-                    const int y = __ldg(W.pad + x), z = __ldg(W.tim + x);
-                    slots[row] = x;
-                    const int d = row - rprev;
-                    if (k == 0) {
-                        m0y = y;
-                        m0z = z;
-                    } else {
-                        if (k == 1) {
-                            abg_init(fy, m0y, y, d);
-                            abg_init(fz, m0z, z, d);
-                        }
-                        for (int j = 0; j < d; j++) {
-                            abg_predict(fy);
-                            abg_predict(fz);
-                        }
-                        abg_update(fy, y);
-                        abg_update(fz, z);
-                    }
-                    rprev = row;
-                    if (k + 1 < len) {
-                        x = W.up[x];
-                        // the next hit is one row further, or two across a row the link skips
-                        if (row + 2 < nr && x >= __ldg(W.bin_off + rowbase + row + 2)) {
-                            slots[row + 1] = -1;
-                            row += 2;
+            }
+            int d = 1;
+            for (int k = 0; k < len; k++) {
+                const int y = __ldg(W.pad + x), z = __ldg(W.tim + x);
+                const int nx = k + 1 < len ? __ldg(link + x) : 0;      // in flight with the coordinates
+                if (out) slots[row] = x;
+                f.hit(y, z, d);
+                z_last = z;
+                if (k + 1 < len) {
+                    x = nx;
+                    if constexpr (SKIP) {
+                        // the next hit is one row on, or two across a row the link skips
+                        if (out) {
+                            d = row + 2 < nr && x >= __ldg(W.bin_off + rowbase + row + 2) ? 2 : 1;
+                            if (d == 2) slots[row + 1] = -1;
                         } else {
-                            row += 1;
+                            d = row >= 1 && x < __ldg(W.bin_off + rowbase + row - 1) ? 2 : 1;
                         }
                     }
-                }
-                row_last = row;
-            }
-            int r1, r0;
-            const int n_out = extend(W, g, fy, fz, rowbase, row_last, +1, slots, &r1);
-            // filter along the chain in descending rows from its last two hits
-            if constexpr (!SKIP) {
-                const int h1 = slots[row_last], h2 = slots[row_last - 1];
-                abg_init(fy, __ldg(W.pad + h1), __ldg(W.pad + h2), 1);
-                abg_init(fz, __ldg(W.tim + h1), __ldg(W.tim + h2), 1);
-                for (int k = len - 2; k >= 0; k--) {
-                    const int h = slots[row0 + k];
-                    abg_predict(fy);
-                    abg_predict(fz);
-                    abg_update(fy, __ldg(W.pad + h));
-                    abg_update(fz, __ldg(W.tim + h));
-                }
-            } else {
-                const int h1 = slots[row_last];
-                int rp = row_last;
-                bool first = true;
-                for (int r = row_last - 1; r >= row0; r--) {
-                    const int h = slots[r];
-                    if (h < 0) continue;
-                    const int d = rp - r;
-                    if (first) {
-                        abg_init(fy, __ldg(W.pad + h1), __ldg(W.pad + h), d);
-                        abg_init(fz, __ldg(W.tim + h1), __ldg(W.tim + h), d);
-                        first = false;
-                    }
-                    for (int j = 0; j < d; j++) {
-                        abg_predict(fy);
-                        abg_predict(fz);
-                    }
-                    abg_update(fy, __ldg(W.pad + h));
-                    abg_update(fz, __ldg(W.tim + h));
-                    rp = r;
+                    row += dir * d;
                 }
             }
-            const int n_in = extend(W, g, fy, fz, rowbase, row0, -1, slots, &r0);
-            W.cand_n[t] = len + n_in + n_out;
-            W.cand_rows[t] = r0 | (r1 << 16);
+            int r_end = row;
+            const bool far = sizeof(T) == 4 && z_last > NARROW_ZHIT;      // stops at its first row
+            const int n = far ? 0 : extend(W, g, f.fy, f.fz, rowbase, row, dir, nr, slots, &r_end);
+            // both threads of the chain add their part to the candidate (len hits and no rows so far)
+            atomicAdd(W.cand_n + t, n);
+            atomicAdd(W.cand_rows + t, out ? r_end << 16 : r_end);
         }
     }
 }
 
 }  // namespace
 
+int follow_narrow(const DevGeom &g) { return g.ymax[g.n_rows - 1] <= NARROW_YMAX && g.zmax <= NARROW_ZMAX; }
+
 void launch_follow(const Work &W, cudaStream_t s) {
     const int block = W.tune.block[3] > 0 ? W.tune.block[3] : 128;
-    const int grid = W.tune.grid[3] > 0 ? W.tune.grid[3] : W.sm_count * 8;
+    const int grid = W.tune.grid[3] > 0 ? W.tune.grid[3] : W.sm_count * FO_CTAS;
     int32_t *perm = W.perm;
     k_follow_order<<<W.sm_count * 8, 256, 0, s>>>(W, perm);
     if (W.rules & TPC_RULE_SKIP_ROW)
-        k_follow<true><<<grid, block, 0, s>>>(W, perm);
+        W.narrow ? k_follow<true, int><<<grid, block, 0, s>>>(W, perm)
+                 : k_follow<true, long long><<<grid, block, 0, s>>>(W, perm);
     else
-        k_follow<false><<<grid, block, 0, s>>>(W, perm);
+        W.narrow ? k_follow<false, int><<<grid, block, 0, s>>>(W, perm)
+                 : k_follow<false, long long><<<grid, block, 0, s>>>(W, perm);
 }
 
 }  // namespace tpc

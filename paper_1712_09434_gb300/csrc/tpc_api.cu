@@ -95,6 +95,7 @@ size_t layout(tpc_ctx *c, char *base) {
     carve(cur, w.bin_cnt, nb + 1);
     carve(cur, w.chain_off, nb + 1);
     carve(cur, w.chain_start, C);
+    carve(cur, w.chain_last, C);
     carve(cur, w.chain_len, C);
     carve(cur, w.chain_bin, C);
     carve(cur, w.cand_n, C);
@@ -168,6 +169,7 @@ Work make_work(const tpc_ctx *c, const tpc_clusters *in, const tpc_tracks *o, co
     w.ns = c->hgeom.n_sectors;
     w.nr = c->hgeom.n_rows;
     w.rules = c->rules;
+    w.narrow = follow_narrow(c->hgeom);
     w.geom = c->dgeom;
     w.sm_count = c->sm_count;
     w.label = o->label;

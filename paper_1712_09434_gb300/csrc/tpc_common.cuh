@@ -75,6 +75,7 @@ struct Work {
     int n_events, n_clusters, nbins;
     int ns, nr;               // sectors, rows (host copies of the geometry)
     int rules;                // TPC_RULE_* bits (0: the plain readings)
+    int narrow;               // the following's filter fits 32-bit words on this geometry
     // outputs
     int32_t *label, *trk_off, *trk_hits, *ev_trk_off, *ndf, *n_tracks;
     float *par, *xref, *cov, *chi2;
@@ -95,7 +96,7 @@ struct Work {
     int32_t *jump4;           // [N] successor four links further
     int32_t *bin_cnt;         // [nbins + 1] chains starting in the bin
     int32_t *chain_off;       // [nbins + 1] exclusive scan of bin_cnt
-    int32_t *chain_start, *chain_len, *chain_bin;   // [cap_chains]
+    int32_t *chain_start, *chain_last, *chain_len, *chain_bin;   // [cap_chains]
     int cap_chains;
     // following (S5)
     int32_t *perm;            // [cap_chains] order in which it takes the chains
@@ -195,6 +196,7 @@ void launch_grid(const Work &W, cudaStream_t s);
 void launch_links(const Work &W, cudaStream_t s);
 void launch_chains(const Work &W, cudaStream_t s);
 void launch_follow(const Work &W, cudaStream_t s);
+int follow_narrow(const DevGeom &g);
 void launch_select(const Work &W, cudaStream_t s);
 void launch_merge(const Work &W, cudaStream_t s);
 void launch_frame_merge(const Work &W, cudaStream_t s);
