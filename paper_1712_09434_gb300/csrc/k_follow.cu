@@ -81,13 +81,13 @@ __device__ __forceinline__ int nearest(const int32_t *yz, const uint16_t *loc, c
         const int hi = e;
         while (a < e) {
             const int mid = (a + e) >> 1;
-            if ((int)(int16_t)(__ldg(yz + mid) & 0xffff) < py - w) a = mid + 1; else e = mid;
+            if (grid_y(__ldg(yz + mid)) < py - w) a = mid + 1; else e = mid;
         }
         for (int i = a; i < hi; i++) {
             const int32_t v = __ldg(yz + i);
-            const int dy = (int)(int16_t)(v & 0xffff) - py;
+            const int dy = grid_y(v) - py;
             if (dy > w) break;
-            const int dz = (int)((uint32_t)v >> 16) - pz;
+            const int dz = grid_z(v) - pz;
             if (abs(dz) > w) continue;
             const int d2 = dy * dy + dz * dz;
             if (d2 < bd || (d2 == bd && d2 <= w2 && __ldg(loc + i) < __ldg(loc + bi))) { bd = d2; bi = i; bv = v; }
@@ -124,8 +124,8 @@ __device__ __forceinline__ int extend(const Work &W, const DevGeom &g, Abg<T> &f
         if (i >= 0) {
             pend = c0 + (int)__ldg(W.gloc + ps + i);
             pend_row = row;
-            abg_update(fy, (int16_t)(v & 0xffff));
-            abg_update(fz, (int)((uint32_t)v >> 16) - Abg<T>::ZB);
+            abg_update(fy, grid_y(v));
+            abg_update(fz, grid_z(v) - Abg<T>::ZB);
             *row_end = row;
             n++;
             misses = 0;

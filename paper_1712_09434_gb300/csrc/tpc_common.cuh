@@ -86,7 +86,7 @@ struct Work {
     // or decreasing, or the offsets do not run from 0 to n_clusters) every cluster in the last bin
     int32_t *bin_ok;
     // workspace: grid (S1)
-    int32_t *gyz;             // [npad] packed (Y & 0xffff) | (Z << 16), slab order
+    int32_t *gyz;             // [npad] packed (Y + 32768) | (Z << 16), slab order
     uint16_t *gloc;           // [npad] row-local cluster index, slab order
     uint16_t *zoff;           // [nbins * ZOFF_STRIDE] row-local slab offsets
     // links (S2)
@@ -154,6 +154,11 @@ __host__ __device__ inline int kept_words(int n_rows) { return (n_rows + 31) / 3
 __host__ __device__ inline int pstart_of(int32_t off, int b) { return ((off + 7) & ~7) + 8 * b; }
 
 #ifdef __CUDACC__
+// grid payload: Y + 32768 in the lower half, Z in the upper
+__device__ __forceinline__ int32_t grid_pack(int y, int z) { return (int32_t)((uint32_t)(y + 32768) | ((uint32_t)z << 16)); }
+__device__ __forceinline__ int grid_y(int32_t v) { return (int)(v & 0xffff) - 32768; }
+__device__ __forceinline__ int grid_z(int32_t v) { return (int)((uint32_t)v >> 16); }
+
 __device__ __forceinline__ void set_status(const Work &W, int bits) { atomicOr(W.status, bits); }
 
 // floor(a / 2^k) for signed a: arithmetic shift (two's complement, CUDA semantics)
