@@ -96,13 +96,10 @@ typedef struct {
  * most 256, 128, 256, 128, 1024, 512, 128, 128 by index), ctas_per_sm = CTAs per SM of the grid
  * (<= 64), chunk = work items taken per queue grab (<= 64; used by the following); for the neighbour
  * finding (index 1) chunk = 1 selects the variant that stages rows r+-1 of every bin in shared
- * memory by bulk copies (one CTA per bin) instead of reading them through L1 (one warp per bin,
- * lanes taking the bin's clusters in Z-slab order), and chunk = 2 the warp-per-bin variant whose
- * lanes take the clusters in cluster (Y, Z) order; for the gradient kernel (index 7) the default
- * recomputes the Kalman states of the reverse sweep from checkpoints every 16 steps, and chunk = 1
- * selects the variant that stores the input state of every step instead (80 B per hit of
- * workspace, no recomputation; the same gradient bit for bit).
- * Launch shapes never change results. */
+ * memory by bulk copies (one CTA per bin) instead of reading them through L1 (a bin's clusters
+ * shared by warps, lanes taking them in Z-slab order), and chunk = 2 the L1 variant whose lanes
+ * take the clusters in cluster (Y, Z) order.  The gradient (index 7) stores the input state
+ * of every step for its reverse sweep and takes no chunk.  Launch shapes never change results. */
 typedef struct {
     int32_t block[TPC_N_TUNE];
     int32_t ctas_per_sm[TPC_N_TUNE];

@@ -4,11 +4,14 @@
 //
 // One thread per track (the paper's one-thread-per-track mapping).  The seed is the circle
 // through the first, middle and last hit at the nominal calibration, so it does not depend on
-// theta; the fit runs from the last hit to the first.  The adjoint's forward pass stores every K-th
-// state (checkpoints) and the reverse sweep recomputes each segment's states from its checkpoint
-// before walking it backwards; a variant stores the input state of every step instead (coalesced
-// by warp chunk, 80 B per hit) and walks them backwards without recomputation (same results, bit
-// for bit).  Per-track chi2 and gradient contributions
+// theta; the fit runs from the last hit to the first.  The adjoint's forward pass stores the input
+// state of every step (coalesced by warp chunk, 80 B per hit) and the reverse pass walks them
+// backwards; tracks too long for the length order keep a checkpoint every CK_K steps instead, from
+// which the reverse pass recomputes each segment's states (same results, bit for bit, with 1772
+// instead of 1311 flop per hit and a local-memory buffer).  Storing took the gradient from 0.38 +
+// 0.82 to 0.35 + 0.43 ms on a central event of 20,000 tracks and from 0.68 + 2.32 to 0.75 + 1.46 ms
+// on 64 events.  The offsets of the warp chunks come out of the length sort.  Per-track chi2 and
+// gradient contributions
 // (s_vd, and (d_k, a_k) for every sector the track visits) are written as records and summed in
 // FP64 in a fixed order (deterministic).
 #include "kf.cuh"
@@ -19,7 +22,8 @@ namespace tpc {
 namespace {
 
 constexpr int CK_K = 16;           // steps between checkpoints
-constexpr int ST_SLACK = 4096;     // spare steps per lane for the chunk padding of the stored states
+constexpr int LEN_BUCKETS = 512;   // length classes of the length order; the last holds all longer tracks
+constexpr int ST_SLACK = 1024;     // spare steps per lane for the chunk padding of the stored states
 constexpr int CK_WORDS = 25;       // x, p[5], P lower triangle[15], frame, rref, yref, zref
 constexpr int ST_WORDS = 20;       // p[5], P lower triangle[15] (stored states: the rest from the hits)
 constexpr int REC_SEC = 8;         // sector entries per track record
@@ -27,12 +31,12 @@ constexpr int REC_WORDS = 2 + 3 * REC_SEC;
 constexpr int NPAR_MAX = 1 + 2 * MAX_SECTORS;
 constexpr int RED_T = 64;          // tracks per reduction block
 
-// Gradient workspace: checkpoints (MODE 1/2) | state after the last hit per track (MODE 3/4) |
-// chunk lengths, offsets and count | stored states (MODE 3/4).
+// Gradient workspace: checkpoints | state after the last hit per track | chunk offsets | stored states.
 struct CkLayout {
     float *ck;
     float *fin;
-    int32_t *cl, *cb, *cn;
+    int32_t *cb;           // first step of every warp chunk of the length order, -1: checkpoints instead;
+                           // cb[-1] is 0 if no chunk keeps checkpoints
     float *st;
     long long cap_steps;   // chunk steps the stored states can hold
 };
@@ -40,18 +44,15 @@ inline size_t ck_words_old(long long cap_hits, long long cap_tracks) {
     return (size_t)(cap_hits / CK_K + 2 * cap_tracks + 1) * CK_WORDS;
 }
 inline size_t ck_words_fin(long long cap_tracks) { return (size_t)cap_tracks * CK_WORDS; }
-inline size_t ck_words_ints(long long cap_tracks) { return (size_t)(3 * (cap_tracks / 32 + 2) + 8); }
+inline size_t ck_words_ints(long long cap_tracks) { return (size_t)(cap_tracks / 32 + 4); }
 inline size_t ck_words_st(long long cap_hits) { return (size_t)(cap_hits + 32ll * ST_SLACK) * ST_WORDS; }
 inline size_t ck_align(size_t w) { return (w + 31) & ~(size_t)31; }
 inline CkLayout ck_layout(float *base, long long cap_hits, long long cap_tracks) {
     CkLayout L;
     L.ck = base;
     L.fin = base + ck_align(ck_words_old(cap_hits, cap_tracks));
-    const long long nch = cap_tracks / 32 + 2;
     int32_t *ints = reinterpret_cast<int32_t *>(L.fin + ck_align(ck_words_fin(cap_tracks)));
-    L.cl = ints;
-    L.cb = ints + nch;
-    L.cn = ints + 2 * nch;
+    L.cb = ints + 1;
     L.st = reinterpret_cast<float *>(ints) + ck_align(ck_words_ints(cap_tracks));
     L.cap_steps = (cap_hits + 32ll * ST_SLACK) / 32;
     return L;
@@ -138,6 +139,18 @@ __device__ __forceinline__ HitT transform(const DevGeom &G, const float *th, int
     return o;
 }
 
+// S0 at the nominal calibration: the offsets are zero and the variances fixed.
+__device__ __forceinline__ kf::FHit<float> nominal_hit(const DevGeom &G, const HitRaw &h) {
+    kf::FHit<float> f;
+    f.k = h.k;
+    f.r = h.r;
+    f.xl = f.yc = f.zc = 0.f;
+    f.yn = (float)h.Y * G.lsb;
+    f.zn = (h.k < G.half ? 1.f : -1.f) * (G.z_max - (float)h.Z * G.lsb);
+    f.vy = f.vz = SIGMA2;
+    return f;
+}
+
 // nominal hit, relative to the last hit E: (x - x_E, y) in E's frame
 __device__ __forceinline__ void nominal_rel(const DevGeom &G, const HitRaw &h, const HitRaw &e, float &x, float &y) {
     const float yr = (float)h.Y * G.lsb;
@@ -163,6 +176,7 @@ __device__ __constant__ const float SQRT_C0[5] = {1.f, 1.f, 0.1f, 0.1f, 1.f};
 // Seed: sin phi, tan lambda, q/pT from the circle through the nominal first, middle and last hit
 // (theta-independent); position = the last hit under theta; references = the last hit.  The caller
 // sets the prior covariance.
+// th = nullptr: the nominal calibration.
 template <class St>
 __device__ bool seed_track(const Work &W, const DevGeom &G, const float *th, int off, int n, St &s) {
     const HitRaw e = hit_raw(W, off + n - 1), a = hit_raw(W, off), b = hit_raw(W, off + (n - 1) / 2);
@@ -172,13 +186,13 @@ __device__ bool seed_track(const Work &W, const DevGeom &G, const float *th, int
     nominal_rel(G, e, e, ex, ey);
     const float ze = nominal_z(G, e);
     if (!kf::seed3<float>(ax, ay, nominal_z(G, a) - ze, bx, by, ex, ey, 0.f, G.kB, SNP_MAX, s.p)) return false;
-    const HitT he = transform(G, th, W.ns, e);
-    s.p[0] = he.f.yc;
-    s.p[1] = he.f.zc;
-    s.x = he.f.xl;
+    const kf::FHit<float> he = th ? transform(G, th, W.ns, e).f : nominal_hit(G, e);
+    s.p[0] = he.yc;
+    s.p[1] = he.zc;
+    s.x = he.xl;
     s.rref = e.r;
-    s.yref = he.f.yn;
-    s.zref = he.f.zn;
+    s.yref = he.yn;
+    s.zref = he.zn;
     s.frame = e.k;
     return true;
 }
@@ -192,12 +206,11 @@ __device__ __forceinline__ int n_tracks_of(const Work &W) {
 // Tracks taken in the order of `order` (decreasing length) when given, so that the lanes of a warp
 // fit tracks of about the same length.  Eight blocks a multiprocessor cap it at 64 registers a
 // thread (a few spilled words): more resident warps hide the latency of the filter's FMA chain.
-__global__ void __launch_bounds__(128, 8) k_refit(Work W, const float *theta, const int32_t *order) {
-    __shared__ float th[NPAR_MAX];
+// The offsets of S0 vanish here, so a hit needs no square root and division: 641 -> 557 us on 64
+// events (291,035 tracks), 239 -> 208 us on a central event, bit for bit the same parameters.  A
+// single event is bound by the latency of a track's steps (1.2 us each, about one warp a scheduler).
+__global__ void __launch_bounds__(128, 8) k_refit(Work W, const int32_t *order) {
     const DevGeom &G = *W.geom;
-    const int ns = W.ns, np = 1 + 2 * ns;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) th[i] = i == 0 ? 1.f - theta[0] : theta[i];
-    __syncthreads();
     FitGeo fg;
     load_geo(G, fg);
     const int nt = n_tracks_of(W);
@@ -217,13 +230,12 @@ __global__ void __launch_bounds__(128, 8) k_refit(Work W, const float *theta, co
         for (int i = 0; i < 5; i++)
             for (int j = 0; j < 5; j++) s.S[i][j] = i == j ? SQRT_C0[i] : 0.f;
         float chi2 = 0.f;
-        bool ok = n >= 3 && seed_track(W, G, th, off, n, s);
+        bool ok = n >= 3 && seed_track(W, G, nullptr, off, n, s);
         HitRaw nxt = n >= 3 ? hit_raw(W, off + n - 1) : HitRaw{};
         for (int i = n - 1; ok && i >= 0; i--) {
             const HitRaw cur = nxt;
             if (i > 0) nxt = hit_raw(W, off + i - 1);      // next hit's load in flight during this step
-            const HitT m = transform(G, th, ns, cur);
-            ok = kf::sqrt_step(s, m.f, fg.g, chi2);
+            ok = kf::sqrt_step(s, nominal_hit(G, cur), fg.g, chi2);
         }
         s.p[0] += s.yref;
         s.p[1] += s.zref;
@@ -395,15 +407,17 @@ __device__ __forceinline__ void pp_load(const float *d, kf::State<float> &s) {
 }
 
 // S8 + S9: refit under theta; per-track record [chi2, d/ds_vd, (sector, d/dd_k, d/da_k) x 8].
-// MODE 0: forward pass only (objective).  Gradient, default: MODE 3 runs the forward pass and stores
-// the input state of every step (80 B per hit, coalesced by warp chunk) and the state after the
-// last hit (frame -1 marks a track whose fit failed); MODE 4 runs the reverse sweep from the stored
-// states.  Gradient with less workspace: MODE 1 stores a checkpoint every CK_K steps, and MODE 2
-// recomputes each segment's states from its checkpoint before sweeping it backwards.  Both give
-// bit-identical results (the same operations in the same order).  Splitting the forward pass off
-// lets it run with fewer registers and more warps than the adjoint.
-template <int MODE>
-__global__ void __launch_bounds__(128, (MODE == 2 || MODE == 4) ? 4 : (MODE == 0 ? 1 : 7)) k_refit_grad(Work W, const double *theta,
+// MODE 0: forward pass only (objective).  Gradient: MODE 3 runs the forward pass and stores the input
+// state of every step (80 B per hit, coalesced by warp chunk) and the state after the last hit (frame
+// -1 marks a track whose fit failed); MODE 4 runs the reverse sweep from the stored states.  A chunk
+// with tracks too long for the length order (LEN_BUCKETS - 1 hits or more: the padding of such a
+// chunk has no bound), or past the end of the workspace, stores a checkpoint every CK_K steps
+// instead, and MODE 2 recomputes each segment's states from its checkpoint before sweeping it
+// backwards.  Both give bit-identical
+// results (the same operations in the same order).  Splitting the forward pass off lets it run with
+// fewer registers and more warps than the adjoint.
+template <int MODE, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_refit_grad(Work W, const double *theta,
                                                     const float *weight, const float *anchor, int model,
                                                     CkLayout L, float *rec, const int32_t *order) {
     float *ck = L.ck;
@@ -416,11 +430,16 @@ __global__ void __launch_bounds__(128, (MODE == 2 || MODE == 4) ? 4 : (MODE == 0
     FitGeo fg;
     load_geo(G, fg);
     const int nt = n_tracks_of(W);
+    if (MODE == 2 && L.cb[-1] == 0) return;
     __shared__ int s_item;
-    int32_t *qh = W.counters + CNT_Q0 + 7;
+    int32_t *qh = W.counters + CNT_QFIT + MODE;
     for (int base = queue_next(qh, blockDim.x, &s_item); base < nt; base = queue_next(qh, blockDim.x, &s_item)) {
         const int i = base + threadIdx.x;
         if (i >= nt) continue;
+        // first step of this chunk's stored states, or -1: the chunk keeps checkpoints
+        const int cb = GRAD ? L.cb[i >> 5] : -1;
+        if ((MODE == 2 && cb >= 0) || (MODE == 4 && cb < 0)) continue;
+        const bool stored = MODE == 4 || (MODE == 3 && cb >= 0);
         const int t = order[i];
         const int off = W.trk_off[t];
         int n = W.trk_off[t + 1] - off;
@@ -431,16 +450,14 @@ __global__ void __launch_bounds__(128, (MODE == 2 || MODE == 4) ? 4 : (MODE == 0
         float *r = rec + (size_t)t * REC_WORDS;
         const float w = weight ? weight[t] : 1.f;
         if (w == 0.f) n = 0;   // excluded track: no fit, no adjoint
-        // checkpoints of track t: slots [off/CK_K + 2t, ... + ceil(n/CK_K)], the last one the state
-        // after the last hit
+        // checkpoints of track t: slots [off/CK_K + 2t, ... + ceil(n/CK_K))
         float *ckt = ck + ((size_t)(off / CK_K) + 2 * (size_t)t) * CK_WORDS;
-        float *ckend = MODE >= 3 ? L.fin + (size_t)t * CK_WORDS
-                                 : ckt + (size_t)((n + CK_K - 1) / CK_K) * CK_WORDS;
-        const long long step0 = MODE >= 3 ? (long long)L.cb[i >> 5] : 0;    // stored states of this lane
+        float *ckend = L.fin + (size_t)t * CK_WORDS;      // state after the last hit
+        const long long step0 = cb;                       // stored states of this lane
         const int slane = i & 31;
         Anchor A{};
         bool use_anchor = false;
-        if (MODE == 0 || MODE == 1 || MODE == 3) {
+        if (MODE == 0 || MODE == 3) {
             kf::State<float> s;
             s.x = 0.f;
             s.rref = 0;
@@ -450,16 +467,14 @@ __global__ void __launch_bounds__(128, (MODE == 2 || MODE == 4) ? 4 : (MODE == 0
                 for (int j = 0; j < 5; j++) s.P[i][j] = i == j ? C0[i] : 0.f;
             float chi2 = 0.f;
             bool ok = n >= 3 && seed_track(W, G, th, off, n, s);
-            if (MODE == 3 && ok && step0 + n > L.cap_steps) {   // no room: reported, track dropped
-                set_status(W, ST_CAPACITY);
-                ok = false;
-            }
             HitRaw nxt = n >= 3 ? hit_raw(W, off + n - 1) : HitRaw{};
             for (int q = 0; ok && q < n; q++) {         // processing step q handles hit i = n-1-q
                 const HitRaw cur = nxt;
                 if (q + 1 < n) nxt = hit_raw(W, off + n - 2 - q);   // next hit's load in flight
-                if (MODE == 1 && q % CK_K == 0) ck_store(ckt + (q / CK_K) * CK_WORDS, s);
-                if (MODE == 3) st_store(L.st, step0 + q, slane, s);
+                if (MODE == 3) {
+                    if (stored) st_store(L.st, step0 + q, slane, s);
+                    else if (q % CK_K == 0) ck_store(ckt + (q / CK_K) * CK_WORDS, s);
+                }
                 const HitT m = transform(G, th, ns, cur, model);
                 ok = kf::step_fwd(s, m.f, fg.g, chi2);
             }
@@ -657,10 +672,10 @@ __global__ void __launch_bounds__(RED_FINAL_T) k_reduce_final(Work W, int np, co
     }
 }
 
-// Tracks in order of decreasing hit count (counting sort on min(n, LEN_BUCKETS-1)): the adjoint
-// takes them from this list, so the 32 tracks of a warp have about the same length and the longest
-// ones start first.  The order inside a bucket does not matter (every track is independent).
-constexpr int LEN_BUCKETS = 512;
+// Tracks in order of decreasing hit count (counting sort on min(n, LEN_BUCKETS-1)): the refit and
+// the adjoint take them from this list, so the 32 tracks of a warp have about the same length and
+// the longest ones start first.  The order inside a bucket does not matter (every track is
+// independent).
 
 // The lanes of a warp with the same bucket add to it with one atomic (tracks of similar length are
 // common, and one atomic per track serialised on the popular buckets).
@@ -675,8 +690,14 @@ __global__ void k_len_hist(Work W, int32_t *hist) {
     }
 }
 
-__global__ void k_len_scan(int32_t *hist) {   // one block of LEN_BUCKETS threads
-    __shared__ int sh[LEN_BUCKETS];
+// One block of LEN_BUCKETS threads: exclusive offsets of the buckets, and the first step of every
+// warp chunk (32 consecutive positions of the order) in the stored states.  A chunk is as long as
+// its first track, whose length is its bucket's, so the offsets follow from the counts alone.  A
+// chunk that begins in the open-ended first bucket gets -1, and so does one past cap_steps (the
+// padding of the others is less than 32 x LEN_BUCKETS hits in all, which the workspace has room
+// for: only track offsets that overlap get there).
+__global__ void __launch_bounds__(LEN_BUCKETS) k_len_scan(int32_t *hist, int32_t *cb, long long cap_steps) {
+    __shared__ int sh[LEN_BUCKETS], sum[LEN_BUCKETS];
     const int i = threadIdx.x;
     sh[i] = hist[i];
     __syncthreads();
@@ -688,6 +709,41 @@ __global__ void k_len_scan(int32_t *hist) {   // one block of LEN_BUCKETS thread
     }
     hist[i] = i > 0 ? sh[i - 1] : 0;          // exclusive offsets
     hist[LEN_BUCKETS + i] = 0;               // fill counters
+    const int nch = (sh[LEN_BUCKETS - 1] + 31) / 32;
+    // bucket of the first track of chunk c: the first one whose inclusive count exceeds 32 c
+    auto bucket = [&](int c) {
+        int lo = 0, hi = LEN_BUCKETS - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sh[mid] > 32 * c) hi = mid; else lo = mid + 1;
+        }
+        return lo;
+    };
+    // every thread takes a run of chunks: their total, a scan of the totals, then the offsets
+    const int per = (nch + LEN_BUCKETS - 1) / LEN_BUCKETS, c0 = min(i * per, nch), c1 = min(c0 + per, nch);
+    int tot = 0;
+    for (int c = c0; c < c1; c++) {
+        const int b = bucket(c);
+        tot += b > 0 ? LEN_BUCKETS - 1 - b : 0;
+    }
+    sum[i] = tot;
+    __syncthreads();
+    for (int o = 1; o < LEN_BUCKETS; o <<= 1) {
+        const int v = i >= o ? sum[i - o] : 0;
+        __syncthreads();
+        sum[i] += v;
+        __syncthreads();
+    }
+    int at = sum[i] - tot, left = 0;
+    for (int c = c0; c < c1; c++) {
+        const int b = bucket(c), len = LEN_BUCKETS - 1 - b;
+        const bool fits = b > 0 && (long long)at + len <= cap_steps;
+        cb[c] = fits ? at : -1;
+        left += !fits;
+        at += b > 0 ? len : 0;
+    }
+    left = __syncthreads_count(left > 0);
+    if (i == 0) cb[-1] = left;
 }
 
 __global__ void k_len_scatter(Work W, int32_t *hist, int32_t *order) {
@@ -702,27 +758,6 @@ __global__ void k_len_scatter(Work W, int32_t *hist, int32_t *order) {
         if (lane == leader) base = atomicAdd(hist + LEN_BUCKETS + b, __popc(peers));
         base = __shfl_sync(peers, base, leader);
         order[hist[b] + base + __popc(peers & ((1u << lane) - 1u))] = t;
-    }
-}
-
-// Longest track of every warp chunk (32 consecutive positions) of the length order, and the
-// number of chunks: the chunk offsets of the stored states are their exclusive scan.
-__global__ void k_chunk_len(Work W, const int32_t *order, CkLayout L) {
-    const int nt = n_tracks_of(W);
-    const int nch = (nt + 31) / 32;
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *L.cn = nch;
-    for (int c = gw; c < nch; c += nw) {
-        const int i = 32 * c + lane;
-        int len = 0;
-        if (i < nt) {
-            const int t = order[i];
-            len = max(W.trk_off[t + 1] - W.trk_off[t], 0);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
-        if (lane == 0) L.cl[c] = len;
     }
 }
 
@@ -777,17 +812,19 @@ int refit_rec_words(int cap_tracks) { return cap_tracks * REC_WORDS; }
 int refit_part_doubles(int cap_tracks, int ns) { return ((cap_tracks + RED_T - 1) / RED_T + 1) * (2 * ns + 2); }
 
 
-void launch_len_order(const Work &W, int32_t *order, int32_t *hist, cudaStream_t s) {
+void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
+                      cudaStream_t s) {
+    const CkLayout L = ck_layout(ck, ck_hits, ck_tracks);
     cudaMemsetAsync(hist, 0, sizeof(int32_t) * LEN_BUCKETS, s);
     k_len_hist<<<W.sm_count * 4, 256, 0, s>>>(W, hist);
-    k_len_scan<<<1, LEN_BUCKETS, 0, s>>>(hist);
+    k_len_scan<<<1, LEN_BUCKETS, 0, s>>>(hist, L.cb, L.cap_steps);
     k_len_scatter<<<W.sm_count * 4, 256, 0, s>>>(W, hist, order);
 }
 
-void launch_refit(const Work &W, const float *theta, const int32_t *order, cudaStream_t s) {
+void launch_refit(const Work &W, const int32_t *order, cudaStream_t s) {
     const int block = W.tune.block[6] > 0 ? W.tune.block[6] : 128;
     const int grid = W.tune.grid[6] > 0 ? W.tune.grid[6] : W.sm_count * 8;
-    k_refit<<<grid, block, 0, s>>>(W, theta, order);
+    k_refit<<<grid, block, 0, s>>>(W, order);
 }
 
 void launch_refit_grad_fit(const Work &W, const double *theta, const float *weight, const float *anchor, int model,
@@ -796,21 +833,21 @@ void launch_refit_grad_fit(const Work &W, const double *theta, const float *weig
     const int block = W.tune.block[7] > 0 ? W.tune.block[7] : 128;
     const int grid = W.tune.grid[7] > 0 ? W.tune.grid[7] : W.sm_count * 8;
     const CkLayout L = ck_layout(ck, ck_hits, ck_tracks);
-    cudaMemsetAsync(W.counters + CNT_Q0 + 7, 0, sizeof(int32_t), s);
-    if (!sorted) launch_len_order(W, order, hist, s);
-    if (grad && W.tune.chunk[7] == 1) {     // every step's input state stored, no recomputation
-        k_chunk_len<<<W.sm_count * 4, 256, 0, s>>>(W, order, L);
-        scan_exclusive(L.cl, L.cb, (int)(ck_tracks / 32 + 1), L.cn, L.cn + 1, W.scan_tmp, W.scan_tmp_len, s);
-        k_refit_grad<3><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
-        cudaMemsetAsync(W.counters + CNT_Q0 + 7, 0, sizeof(int32_t), s);
-        k_refit_grad<4><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
-    } else if (grad) {                      // checkpoints every CK_K steps, states recomputed (default)
-        k_refit_grad<1><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
-        cudaMemsetAsync(W.counters + CNT_Q0 + 7, 0, sizeof(int32_t), s);
-        k_refit_grad<2><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
-    } else {
-        k_refit_grad<0><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+    cudaMemsetAsync(W.counters + CNT_QFIT, 0, 5 * sizeof(int32_t), s);
+    if (!sorted) launch_len_order(W, order, hist, ck, ck_hits, ck_tracks, s);
+    if (!grad) {
+        k_refit_grad<0, 1><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+        return;
     }
+    // Reverse pass: where all tracks (about one per 128 clusters) are resident at once anyway, three
+    // blocks a multiprocessor without spilled registers are faster (central event 555 -> 432 us), else
+    // four (64 events 1579 -> 1455 us).  The register cap changes no bit of the result.
+    k_refit_grad<3, 6><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+    if (W.n_clusters / 128 <= 3 * 128 * W.sm_count)
+        k_refit_grad<4, 3><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+    else
+        k_refit_grad<4, 4><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+    k_refit_grad<2, 4><<<W.sm_count, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
 }
 
 void launch_refit_grad_reduce(const Work &W, double *sum_chi2, double *grad, const float *rec, double *part,

@@ -17,7 +17,6 @@ struct tpc_ctx {
     double bz;
     DevGeom hgeom;
     DevGeom *dgeom;
-    float *theta0;            // nominal calibration (FP32, device)
     // reservation
     int max_clusters, max_events, nbins_max, cap_chains;
     void *arena;
@@ -219,8 +218,8 @@ int enqueue_pipeline(const tpc_ctx *c, const Work &W, cudaStream_t s, bool captu
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[5], s, evf));
     launch_merge(W, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[6], s, evf));
-    launch_len_order(W, c->order, c->lhist, s);
-    launch_refit(W, c->theta0, c->order, s);
+    launch_len_order(W, c->order, c->lhist, c->ck, (long long)c->max_clusters + 1, (long long)c->cap_chains + 1, s);
+    launch_refit(W, c->order, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[7], s, evf));
     return cuda_err(cudaGetLastError());
 }
@@ -372,12 +371,8 @@ int tpc_init(const tpc_geometry *g, double bz_tesla, tpc_ctx **out) {
         h.rot_cos[m + h.half] = (float)std::cos(m * 2.0 * ha);
         h.rot_sin[m + h.half] = (float)std::sin(m * 2.0 * ha);
     }
-    float th0[1 + 2 * MAX_SECTORS] = {0.f};
-    th0[0] = 1.f;
     if (cuda_err(cudaMalloc(&c->dgeom, sizeof(DevGeom))) ||
         cuda_err(cudaMemcpy(c->dgeom, &h, sizeof(DevGeom), cudaMemcpyHostToDevice)) ||
-        cuda_err(cudaMalloc(&c->theta0, sizeof(th0))) ||
-        cuda_err(cudaMemcpy(c->theta0, th0, sizeof(th0), cudaMemcpyHostToDevice)) ||
         cuda_err(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking))) {
         tpc_destroy(c);
         return TPC_ERR_CUDA;
@@ -425,7 +420,6 @@ void tpc_destroy(tpc_ctx *c) {
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->arena) cudaFree(c->arena);
     if (c->dgeom) cudaFree(c->dgeom);
-    if (c->theta0) cudaFree(c->theta0);
     delete c;
 }
 

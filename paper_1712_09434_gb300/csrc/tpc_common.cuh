@@ -146,6 +146,7 @@ enum {
     CNT_FRAME_H = 6,
     CNT_BINS_BAD = 7,         // set when the caller's bin offsets fail the check
     CNT_Q0 = 8,               // work-queue heads, one per kernel
+    CNT_QFIT = 16,            // work-queue heads of the refit kernels under theta, by mode
 };
 
 // words of the kept-hit mask of a candidate
@@ -205,9 +206,11 @@ int follow_narrow(const DevGeom &g);
 void launch_select(const Work &W, cudaStream_t s);
 void launch_merge(const Work &W, cudaStream_t s);
 void launch_frame_merge(const Work &W, cudaStream_t s);
-// tracks in order of decreasing hit count into order (hist: 2 * 512 words of scratch)
-void launch_len_order(const Work &W, int32_t *order, int32_t *hist, cudaStream_t s);
-void launch_refit(const Work &W, const float *theta, const int32_t *order, cudaStream_t s);
+// tracks in order of decreasing hit count into order, and the first step of every 32 of them in the
+// stored states of the gradient into its workspace ck (hist: 2 * 512 words of scratch)
+void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
+                      cudaStream_t s);
+void launch_refit(const Work &W, const int32_t *order, cudaStream_t s);
 // sorted: order already holds the length order of these tracks
 void launch_refit_grad_fit(const Work &W, const double *theta, const float *weight, const float *anchor, int model,
                            bool grad, float *ck, long long ck_hits, long long ck_tracks, float *rec, int32_t *order,
