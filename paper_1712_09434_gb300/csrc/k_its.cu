@@ -5,10 +5,18 @@
 // and their errors) is expressed in the same frame (y = 0, sin phi = sin(phi0 - alpha_k)).  The
 // drift calibration is what the match is for, so z only has to fall in a loose window; the match
 // chi2 is over (y, sin phi, tan lambda, q/pT) with the TPC covariance plus the ITS errors.  Each side
-// keeps its best partner by (floor(chi2 * 2^20), index) (64-bit atomicMin on the ITS side); mutual
-// best pairs are matched, and a matched track that starts within the first 8 pad rows, has at least
+// keeps its best partner by (floor(chi2 * 2^20), index) (64-bit atomicMin); mutual best pairs are
+// matched, and a matched track that starts within the first 8 pad rows, has at least
 // 30 hits and |sin phi| < 0.9 at the vertex gets the ITS track's values as its references at the
 // vertex (the anchor input of tpc_refit_grad).
+//
+// What bounds it: FP64, of which this chip has little, and a warp pays for a test however few of its
+// lanes are in it.  So the work is split by kind: a
+// thread per track for the FP64 step to the vertex; eight lanes a track that pass over the ITS
+// tracks of its window in FP32, with margins, and list the pairs that are left (a few per track); a
+// thread per listed pair for the FP64 test, so that all lanes of a warp have one.  In one kernel,
+// with a thread per track for all of it, almost every candidate of a warp had some lane in the FP64
+// test: 766 us on a central event (25,762 x 19,400 tracks); now 22 + 58 + 22 us.
 #include "kf.cuh"
 #include "tpc_common.cuh"
 
@@ -46,18 +54,27 @@ __device__ __forceinline__ int phi_bin(double phi) {
     return b < 0 ? b + ITS_NPHI : b;
 }
 
+constexpr int ITS_REC = 18;      // doubles per track: y, z, snp, tl, q/pT, 4x4 covariance (10), phi, sin, cos alpha
+constexpr int ITS_LANES = 8;     // lanes a track takes its window with
+
 struct ItsArgs {
     const float *its;          // [n_its][8]
     int n_its;
     int32_t *match_trk, *match_its;
     float *anchor;             // [n_tracks][8] or nullptr
     double kB, alpha0, dalpha; // curvature constant, sector k centre angle = alpha0 + (k mod half) dalpha
-    int32_t *cnt, *off, *fill, *list, *sec;   // sec: 1 if the track may carry references
+    int32_t *cnt, *off, *fill, *sec;   // sec: 1 if the track may carry references
     unsigned long long *best_trk, *best_its;
     double *sc;                // [n_its][2] sin, cos of phi0
+    float4 *srt;               // [n_its][3] ITS tracks in bin order: phi, z, tl, q/pT | s_phi, s_tl, s_q, index | sin, cos
+    double *rec;               // [nt_cap][ITS_REC] tracks at the vertex
+    int2 *pairs;               // [cap_pairs] (track, ITS track) left for the FP64 test
+    int32_t *n_pairs;
+    int cap_pairs;
 };
 
 __global__ void k_its_count(Work W, ItsArgs A) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *A.n_pairs = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n_its; i += gridDim.x * blockDim.x) {
         const double phi = A.its[8 * (size_t)i];
         atomicAdd(A.cnt + phi_bin(phi) * ITS_NTL + tl_bin(A.its[8 * (size_t)i + 2]), 1);
@@ -70,8 +87,12 @@ __global__ void k_its_count(Work W, ItsArgs A) {
 
 __global__ void k_its_fill(Work W, ItsArgs A) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n_its; i += gridDim.x * blockDim.x) {
-        const int b = phi_bin(A.its[8 * (size_t)i]) * ITS_NTL + tl_bin(A.its[8 * (size_t)i + 2]);
-        A.list[A.off[b] + atomicAdd(A.fill + b, 1)] = i;
+        const float *r = A.its + 8 * (size_t)i;
+        const int b = phi_bin(r[0]) * ITS_NTL + tl_bin(r[2]);
+        float4 *d = A.srt + 3 * (size_t)(A.off[b] + atomicAdd(A.fill + b, 1));
+        d[0] = make_float4(r[0], r[1], r[2], r[3]);
+        d[1] = make_float4(r[4], r[6], r[7], __int_as_float(i));
+        d[2] = make_float4((float)A.sc[2 * (size_t)i], (float)A.sc[2 * (size_t)i + 1], 0.f, 0.f);
     }
 }
 
@@ -100,10 +121,38 @@ __device__ double chi2_4(double M[4][4], const double d[4]) {
     return c2;
 }
 
-// Thread per TPC track: its state at the vertex, then the ITS tracks of the (azimuth, tan lambda)
-// bins that reach into the window; the best (key, ITS index) kept, (key, track) offered to the ITS
-// track.
-__global__ void k_its_match(Work W, ItsArgs A) {
+// The FP64 test of track t (record r) against ITS track i: offers (key, ITS index) to the track and
+// (key, track) to the ITS track.
+__device__ void its_pair(const ItsArgs &A, int t, int i) {
+    const double *q = A.rec + (size_t)t * ITS_REC;
+    const float *r = A.its + 8 * (size_t)i;
+    const double phi_t = q[15], sa = q[16], ca = q[17];
+    if (fabs(wrap_pi((double)r[0] - phi_t)) > ITS_DPHI) return;
+    if (fabs((double)r[2] - q[3]) > ITS_DTL || fabs((double)r[1] - q[1]) > ITS_DZ) return;
+    // sin, cos of phi0 - alpha from those of phi0 and alpha (no transcendental per pair)
+    const double s0 = A.sc[2 * (size_t)i], c0 = A.sc[2 * (size_t)i + 1];
+    const double sdp = s0 * ca - c0 * sa, cdp = c0 * ca + s0 * sa;
+    const double d[4] = {q[0], q[2] - sdp, q[3] - (double)r[2], q[4] - (double)r[3]};
+    const double cph = cdp * (double)r[4];
+    const double ev[4] = {ITS_SIGMA_Y * ITS_SIGMA_Y, cph * cph, (double)r[6] * r[6], (double)r[7] * r[7]};
+    double M[4][4];
+    for (int a = 0, m = 5; a < 4; a++)
+        for (int c = 0; c <= a; c++, m++) M[a][c] = M[c][a] = q[m] + (a == c ? ev[a] : 0.0);
+    // d^T M^-1 d >= d_a^2 / M_aa for a positive definite M (Cauchy-Schwarz): one component beyond the
+    // gate on its own, with a margin far above the rounding of the factorisation, rejects the pair
+    // without it (the same decision)
+    bool beyond = false;
+    for (int a = 0; a < 4; a++) beyond |= d[a] * d[a] > ITS_CHI2 * M[a][a] * (1.0 + 1e-9);
+    if (beyond) return;
+    const double c2 = chi2_4(M, d);
+    if (c2 < 0.0 || c2 > ITS_CHI2) return;
+    const unsigned long long k = (unsigned long long)floor(c2 * 1048576.0) << 32;
+    atomicMin(A.best_trk + t, k | (unsigned)i);
+    atomicMin(A.best_its + i, k | (unsigned)t);
+}
+
+// Thread per TPC track: its state and covariance at the vertex in FP64.
+__global__ void k_its_state(Work W, ItsArgs A) {
     const DevGeom &g = *W.geom;
     const int nt = min(*W.n_tracks, W.cap_tracks);
     const int nbe = W.ns * W.nr;
@@ -136,70 +185,67 @@ __global__ void k_its_match(Work W, ItsArgs A) {
         if (!kf::prop_fwd<double>(s, -s.x, A.kB, (double)SNP_MAX)) continue;
         A.sec[t] = first_row <= REF_MAX_FIRST_ROW && n_hits >= REF_MIN_HITS && fabs(s.p[2]) < REF_MAX_SNP;
         const double alpha = A.alpha0 + (k % g.half) * A.dalpha;
-        const double phi_t = alpha + asin(s.p[2]);
-        const double sa = sin(alpha), ca = cos(alpha);
-        const float tl32 = (float)s.p[3], z32 = (float)s.p[1];
-        // FP32 copies for the pre-checks below
-        const float phi32 = (float)phi_t, sa32 = (float)sa, ca32 = (float)ca;
-        const float d0_32 = (float)s.p[0], sn32 = (float)s.p[2], q32 = (float)s.p[4];
-        const float m0_32 = (float)(s.P[0][0] + ITS_SIGMA_Y * ITS_SIGMA_Y), pss32 = (float)s.P[2][2];
-        const float ptt32 = (float)s.P[3][3], pqq32 = (float)s.P[4][4];
         const int ix[4] = {0, 2, 3, 4};
-        unsigned long long best = ~0ull;
+        double *q = A.rec + (size_t)t * ITS_REC;
+        for (int i = 0; i < 5; i++) q[i] = s.p[i];
+        for (int a = 0, m = 5; a < 4; a++)
+            for (int c = 0; c <= a; c++, m++) q[m] = s.P[ix[a]][ix[c]];
+        q[15] = alpha + asin(s.p[2]);
+        q[16] = sin(alpha);
+        q[17] = cos(alpha);
+    }
+}
+
+// ITS_LANES lanes per track over the ITS tracks of the (azimuth, tan lambda) bins that reach into the
+// window; the pairs that the FP32 pre-checks leave go to the list (tested here if it is full).
+__global__ void __launch_bounds__(128) k_its_scan(Work W, ItsArgs A) {
+    const int nt = min(*W.n_tracks, W.cap_tracks);
+    const int sub = threadIdx.x % ITS_LANES;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) / ITS_LANES; t < nt;
+         t += gridDim.x * blockDim.x / ITS_LANES) {
+        if (A.sec[t] < 0) continue;
+        const double *q = A.rec + (size_t)t * ITS_REC;
+        const double phi_t = q[15];
+        const float tl32 = (float)q[3], z32 = (float)q[1], phi32 = (float)phi_t, sa32 = (float)q[16], ca32 = (float)q[17];
+        const float d0_32 = (float)q[0], sn32 = (float)q[2], q32 = (float)q[4];
+        const float m0_32 = (float)(q[5] + ITS_SIGMA_Y * ITS_SIGMA_Y), pss32 = (float)q[7];
+        const float ptt32 = (float)q[10], pqq32 = (float)q[14];
+        const float g = (float)ITS_CHI2 * 1.001f;
+        if (d0_32 * d0_32 > g * m0_32) continue;
         const int b0 = (int)floor((phi_t - ITS_DPHI) / TWO_PI * ITS_NPHI), b1 = (int)floor((phi_t + ITS_DPHI) / TWO_PI * ITS_NPHI);
+        // the tan lambda bins that can hold an ITS track within the window (and its margin)
+        const int tb0 = tl_bin(tl32 - (float)ITS_DTL - 2e-3f), tb1 = tl_bin(tl32 + (float)ITS_DTL + 2e-3f) + 1;
         for (int bb = b0; bb <= b1; bb++) {
             const int bp = ((bb % ITS_NPHI) + ITS_NPHI) % ITS_NPHI;
-            // the tan lambda bins that can hold an ITS track within the window (and its margin)
-            const int j0 = A.off[bp * ITS_NTL + tl_bin(tl32 - (float)ITS_DTL - 2e-3f)];
-            const int j1 = A.off[bp * ITS_NTL + tl_bin(tl32 + (float)ITS_DTL + 2e-3f) + 1];
-            for (int j = j0; j < j1; j++) {
-                const int i = A.list[j];
-                const float *r = A.its + 8 * (size_t)i;
-                // FP32 pre-checks with a margin that the exact tests below can only narrow
-                if (fabsf(r[2] - tl32) > (float)ITS_DTL + 1e-3f || fabsf(r[1] - z32) > (float)ITS_DZ + 1e-3f) continue;
-                {
-                    // the azimuth window and the one-component chi2 bound below, in FP32 with margins
-                    // (1e-3 rad; 0.1 % of the bound) far above FP32 rounding: they only reject pairs
-                    // that the FP64 tests reject too
-                    float dph = r[0] - phi32;
-                    dph -= rintf(dph * (float)(1.0 / TWO_PI)) * (float)TWO_PI;
-                    if (fabsf(dph) > (float)ITS_DPHI + 1e-3f) continue;
-                    const float s0 = (float)A.sc[2 * (size_t)i], c0 = (float)A.sc[2 * (size_t)i + 1];
-                    const float sdp = s0 * ca32 - c0 * sa32, cph = (c0 * ca32 + s0 * sa32) * r[4];
-                    const float d1 = sn32 - sdp, d2 = tl32 - r[2], d3 = q32 - r[3];
-                    const float g = (float)ITS_CHI2 * 1.001f;
-                    if (d0_32 * d0_32 > g * m0_32 || d1 * d1 > g * (pss32 + cph * cph) ||
-                        d2 * d2 > g * (ptt32 + r[6] * r[6]) || d3 * d3 > g * (pqq32 + r[7] * r[7]))
-                        continue;
-                }
-                if (fabs(wrap_pi((double)r[0] - phi_t)) > ITS_DPHI) continue;
-                if (fabs((double)r[2] - s.p[3]) > ITS_DTL || fabs((double)r[1] - s.p[1]) > ITS_DZ) continue;
-                // sin, cos of phi0 - alpha from those of phi0 and alpha (no transcendental per pair)
-                const double s0 = A.sc[2 * (size_t)i], c0 = A.sc[2 * (size_t)i + 1];
-                const double sdp = s0 * ca - c0 * sa, cdp = c0 * ca + s0 * sa;
-                const double d[4] = {s.p[0], s.p[2] - sdp, s.p[3] - (double)r[2], s.p[4] - (double)r[3]};
-                const double cph = cdp * (double)r[4];
-                const double ev[4] = {ITS_SIGMA_Y * ITS_SIGMA_Y, cph * cph, (double)r[6] * r[6], (double)r[7] * r[7]};
-                // d^T M^-1 d >= d_a^2 / M_aa for a positive definite M (Cauchy-Schwarz): one component
-                // beyond the gate on its own, with a margin far above the rounding of the
-                // factorisation, rejects the pair without it (the same decision)
-                bool beyond = false;
-                for (int a = 0; a < 4; a++)
-                    beyond |= d[a] * d[a] > ITS_CHI2 * (s.P[ix[a]][ix[a]] + ev[a]) * (1.0 + 1e-9);
-                if (beyond) continue;
-                double M[4][4];
-                for (int a = 0; a < 4; a++)
-                    for (int c = 0; c < 4; c++) M[a][c] = s.P[ix[a]][ix[c]] + (a == c ? ev[a] : 0.0);
-                const double c2 = chi2_4(M, d);
-                if (c2 < 0.0 || c2 > ITS_CHI2) continue;
-                const unsigned long long q = (unsigned long long)floor(c2 * 1048576.0);
-                const unsigned long long kt = (q << 32) | (unsigned)i;
-                best = kt < best ? kt : best;
-                atomicMin(A.best_its + i, (q << 32) | (unsigned)t);
+            const int j1 = A.off[bp * ITS_NTL + tb1];
+            for (int j = A.off[bp * ITS_NTL + tb0] + sub; j < j1; j += ITS_LANES) {
+                // FP32 pre-checks with margins far above FP32 rounding (1e-3 in tan lambda and z, 1e-3
+                // rad, 0.1 % of the one-component chi2 bound): they only reject pairs that the FP64
+                // tests reject too
+                const float4 r = A.srt[3 * (size_t)j], e = A.srt[3 * (size_t)j + 1], sc = A.srt[3 * (size_t)j + 2];
+                if (fabsf(r.z - tl32) > (float)ITS_DTL + 1e-3f || fabsf(r.y - z32) > (float)ITS_DZ + 1e-3f) continue;
+                float dph = r.x - phi32;
+                dph -= rintf(dph * (float)(1.0 / TWO_PI)) * (float)TWO_PI;
+                if (fabsf(dph) > (float)ITS_DPHI + 1e-3f) continue;
+                const float sdp = sc.x * ca32 - sc.y * sa32, cph = (sc.y * ca32 + sc.x * sa32) * e.x;
+                const float d1 = sn32 - sdp, d2 = tl32 - r.z, d3 = q32 - r.w;
+                if (d1 * d1 > g * (pss32 + cph * cph) || d2 * d2 > g * (ptt32 + e.y * e.y) ||
+                    d3 * d3 > g * (pqq32 + e.z * e.z))
+                    continue;
+                const int i = __float_as_int(e.w);
+                // (a full list is not counted on: the count stays near its capacity)
+                const int p = __ldcg(A.n_pairs) < A.cap_pairs ? atomicAdd(A.n_pairs, 1) : A.cap_pairs;
+                if (p < A.cap_pairs) A.pairs[p] = make_int2(t, i);
+                else its_pair(A, t, i);
             }
         }
-        A.best_trk[t] = best;
     }
+}
+
+__global__ void __launch_bounds__(128) k_its_pairs(ItsArgs A) {
+    const int n = min(*A.n_pairs, A.cap_pairs);
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x)
+        its_pair(A, A.pairs[p].x, A.pairs[p].y);
 }
 
 __global__ void k_its_link(Work W, ItsArgs A) {
@@ -239,7 +285,8 @@ int its_constants(double *out) {
 }
 
 void launch_its_match(const Work &W, const float *its, int n_its, int32_t *match_trk, int32_t *match_its,
-                      float *anchor, double kB, double alpha0, double dalpha, cudaStream_t s) {
+                      float *anchor, double kB, double alpha0, double dalpha, float *scratch, size_t scratch_words,
+                      cudaStream_t s) {
     ItsArgs A;
     A.its = its;
     A.n_its = n_its;
@@ -250,22 +297,33 @@ void launch_its_match(const Work &W, const float *its, int n_its, int32_t *match
     A.alpha0 = alpha0;
     A.dalpha = dalpha;
     // workspace of the tracking, free between calls: counts, offsets and fill levels of the azimuth
-    // bins, the ITS tracks sorted by bin, the first-hit sector of every track, the best keys
+    // bins, the first-hit sector of every track, the best keys
     A.cnt = W.bin_cnt;
     A.off = W.mrg_off;
     A.fill = W.chain_off;
-    A.list = W.mrg_list;
     A.sec = W.trk_n;
     A.best_trk = W.gap_bestT;
     A.best_its = W.gap_bestS;
     A.sc = reinterpret_cast<double *>(W.gap_state);   // 6 words per chain slot >= 2 doubles per ITS track
+    // and the workspace of the refit: track records, the sorted ITS tracks, the pair list in the rest
+    A.n_pairs = W.counters + CNT_ITS_PAIRS;
+    A.rec = reinterpret_cast<double *>(scratch);
+    size_t used = (size_t)W.cap_tracks * ITS_REC * 2;
+    used = (used + 63) & ~(size_t)63;
+    A.srt = reinterpret_cast<float4 *>(scratch + used);
+    used += (size_t)n_its * 12;
+    A.pairs = reinterpret_cast<int2 *>(scratch + used);
+    const size_t left = used < scratch_words ? (scratch_words - used) / 2 : 0;
+    A.cap_pairs = (int)(left < (1u << 30) ? left : (1u << 30));
     const int grid = W.sm_count * 4;
     cudaMemsetAsync(A.cnt, 0, sizeof(int32_t) * (ITS_NBINS + 1), s);
     cudaMemsetAsync(A.fill, 0, sizeof(int32_t) * (ITS_NBINS + 1), s);
     k_its_count<<<grid, 256, 0, s>>>(W, A);
     scan_exclusive(A.cnt, A.off, ITS_NBINS, nullptr, nullptr, W.scan_tmp, W.scan_tmp_len, s);
     k_its_fill<<<grid, 256, 0, s>>>(W, A);
-    k_its_match<<<grid, 128, 0, s>>>(W, A);
+    k_its_state<<<grid, 128, 0, s>>>(W, A);
+    k_its_scan<<<W.sm_count * 12, 128, 0, s>>>(W, A);
+    k_its_pairs<<<grid, 128, 0, s>>>(A);
     k_its_link<<<grid, 256, 0, s>>>(W, A);
 }
 

@@ -508,7 +508,8 @@ int tpc_its_match(tpc_ctx *c, const tpc_clusters *in, const tpc_tracks *trk, con
     TPC_CUDA(cudaMemsetAsync(W.counters + CNT_BINS_BAD, 0, sizeof(int32_t), s));
     launch_bins_check(W, s);
     const double ha = c->geom.half_angle_deg * M_PI / 180.0;
-    launch_its_match(W, its, n_its, match_trk, match_its, anchor, -0.299792458e-2 * c->bz, ha, 2.0 * ha, s);
+    launch_its_match(W, its, n_its, match_trk, match_its, anchor, -0.299792458e-2 * c->bz, ha, 2.0 * ha, c->ck,
+                     refit_ck_words((long long)c->max_clusters + 1, (long long)c->cap_chains + 1), s);
     return cuda_err(cudaGetLastError());
 }
 

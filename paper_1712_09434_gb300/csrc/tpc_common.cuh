@@ -146,6 +146,7 @@ enum {
     CNT_FRAME_H = 6,
     CNT_BINS_BAD = 7,         // set when the caller's bin offsets fail the check
     CNT_Q0 = 8,               // work-queue heads, one per kernel
+    CNT_ITS_PAIRS = 24,       // pairs left for the FP64 test of the ITS matching
     CNT_QFIT = 16,            // work-queue heads of the refit kernels under theta, by mode
 };
 
@@ -222,7 +223,8 @@ int refit_rec_words(int cap_tracks);
 int refit_part_doubles(int cap_tracks, int ns);
 void launch_pack_hits(const Work &W, cudaStream_t s);
 void launch_its_match(const Work &W, const float *its, int n_its, int32_t *match_trk, int32_t *match_its,
-                      float *anchor, double kB, double alpha0, double dalpha, cudaStream_t s);
+                      float *anchor, double kB, double alpha0, double dalpha, float *scratch, size_t scratch_words,
+                      cudaStream_t s);
 int its_match_nphi();
 void launch_looper_pairs(const Work &W, int32_t *pair, int32_t *leg, double kB, double alpha0, double dalpha,
                          double *rec, int nt_cap, cudaStream_t s);
