@@ -76,7 +76,12 @@ __global__ void k_merge_ends(Work W) {
 }
 
 // Accepted segments listed per (event, sector, row of the first kept hit): the merge only looks at
-// segments whose first row lies inside the extrapolation reach.
+// segments whose first row lies inside the extrapolation reach, and reads their first hits (Xtab, Y,
+// Z, index) in that order.
+__device__ __forceinline__ int4 *merge_firsts(const Work &W) {
+    // behind the list of outer ends, in the packed track hits (written later)
+    return reinterpret_cast<int4 *>(W.trk_pack + ((2 * (size_t)W.cap_chains + 3) & ~(size_t)3));
+}
 __global__ void k_merge_fill(Work W) {
     const int n = n_chains_of(W);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -89,7 +94,9 @@ __global__ void k_merge_fill(Work W) {
             if (W.geom->xtab[mid] < e.x) lo = mid + 1; else hi = mid;
         }
         const int b = bin0 + lo;
-        W.mrg_list[W.mrg_off[b] + atomicAdd(W.bin_cnt + b, 1)] = t;
+        const int p = W.mrg_off[b] + atomicAdd(W.bin_cnt + b, 1);
+        W.mrg_list[p] = t;
+        merge_firsts(W)[p] = make_int4(e.x, e.y, e.z, t);
     }
 }
 
@@ -240,78 +247,122 @@ __global__ void k_gap_link(Work W) {
     }
 }
 
-// One warp per outer end S: the lanes take the candidate segments T of the reachable rows of both
-// adjacent sectors 32 at a time; the warp keeps the minimum (D, T) for S and every valid pair offers
-// (D, S) to T with a 64-bit atomicMin.
-__global__ void k_merge_match(Work W) {
-    const DevGeom &g = *W.geom;
-    const int n = n_chains_of(W);
+// The outer end of segment S in the frame of the adjacent sector on side k (0: the next, 1: the
+// previous one).
+struct OuterEnd {
+    long long x1, y1, x2, y2, dxs;
+    int z1, dz, kt;        // Z of the inner point, Z difference, sector
+};
+__device__ __forceinline__ bool outer_end(const Work &W, const DevGeom &g, int s, int k, OuterEnd &o) {
     const int half = W.ns / 2;
+    const int4 p1 = W.outend[2 * s], p2 = W.outend[2 * s + 1];
+    const int ks = p1.w;
+    const int side0 = ks < half ? 0 : half;
+    const int sgn = k == 0 ? +1 : -1;
+    o.kt = side0 + ((ks - side0) + (k == 0 ? 1 : half - 1)) % half;
+    if (k == 1 && o.kt == side0 + ((ks - side0) + 1) % half) return false;   // tiny geometries
+    const long long X1 = p1.x, Y1 = p1.y, X2 = p2.x, Y2 = p2.y;
+    o.x1 = (X1 * g.c30 + sgn * Y1 * g.s30) >> 30;
+    o.y1 = (-sgn * X1 * g.s30 + Y1 * g.c30) >> 30;
+    o.x2 = (X2 * g.c30 + sgn * Y2 * g.s30) >> 30;
+    o.y2 = (-sgn * X2 * g.s30 + Y2 * g.c30) >> 30;
+    o.dxs = o.x2 - o.x1;
+    o.z1 = p1.z;
+    o.dz = p2.z - p1.z;
+    return o.dxs > 0;
+}
+
+// Thread per (outer end, adjacent sector): lists those that can match anything.  The extrapolated Y
+// is monotonic in XT, so its range over the reach |XT - x2| <= MERGE_XMAX is that of the two ends.
+// If the window around it misses the range of the first-hit Y of every segment of that sector, no T
+// there can match (the usual case: S ends away from the edge that faces it).  This decision is the
+// same for all T, so it is taken with full warps here and not by each lane of the warps that match.
+// With the first hits read in bucket order and tested in FP32 before the 64-bit arithmetic, both
+// kernels take 494 us on 64 events (923 as one), 67 us on a central event (170).
+__global__ void __launch_bounds__(128) k_merge_probe(Work W, int32_t *list) {
+    const DevGeom &g = *W.geom;
+    const long long n2 = 2ll * n_chains_of(W);
+    const int lane = threadIdx.x & 31;
+    const bool gap = (W.rules & TPC_RULE_GAP_MERGE) != 0;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n2; i0 += stride) {
+        const long long i = i0 + lane;
+        const int s = (int)(i >> 1), k = (int)(i & 1);
+        bool keep = false;
+        if (i < n2 && W.seg_n[s] >= N_MIN && !(gap && W.next[s] >= 0)) {    // a gap successor: no outer end
+            OuterEnd o;
+            if (outer_end(W, g, s, k, o)) {
+                const long long ya = o.y1 + floor_div_pos((o.x2 - MERGE_XMAX - o.x1) * (o.y2 - o.y1), o.dxs);
+                const long long yb = o.y1 + floor_div_pos((o.x2 + MERGE_XMAX - o.x1) * (o.y2 - o.y1), o.dxs);
+                const long long ymin = ya < yb ? ya : yb, ymx = ya < yb ? yb : ya;
+                const long long bound = W.sec_ymax[W.chain_bin[s] / (W.ns * W.nr) * W.ns + o.kt];
+                keep = !(ymin - W_MERGE > bound || ymx + W_MERGE < -bound);
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (!m) continue;
+        int p = 0;
+        if (lane == 0) p = atomicAdd(W.counters + CNT_MERGE, __popc(m));
+        p = __shfl_sync(0xffffffffu, p, 0);
+        if (keep) list[p + __popc(m & ((1u << lane) - 1u))] = (int32_t)((uint32_t)s << 1 | (uint32_t)k);
+    }
+}
+
+// One warp per listed outer end S and adjacent sector: the lanes take the candidate segments T of the
+// reachable rows 32 at a time; every valid pair offers (D, T) to S and (D, S) to T with 64-bit
+// atomicMin (for S once per warp).
+__global__ void __launch_bounds__(128) k_merge_match(Work W, const int32_t *list) {
+    const DevGeom &g = *W.geom;
+    const int n = W.counters[CNT_MERGE];
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     const float pitch = (float)(g.xtab[W.nr - 1] - g.xtab[0]) / (float)(W.nr - 1);
     const bool gap = (W.rules & TPC_RULE_GAP_MERGE) != 0;
-    for (int s = gw; s < n; s += nw) {
-        if (W.seg_n[s] < N_MIN || (gap && W.next[s] >= 0)) continue;   // a gap successor: no outer end
-        const int4 p1 = W.outend[2 * s], p2 = W.outend[2 * s + 1];
-        const int ks = p1.w;
-        const int ev = W.chain_bin[s] / (W.ns * W.nr);
-        const int side0 = ks < half ? 0 : half;
+    for (int q = gw; q < n; q += nw) {
+        const int s = (int)((uint32_t)list[q] >> 1);
+        OuterEnd o;
+        outer_end(W, g, s, list[q] & 1, o);
+        const int b0 = (W.chain_bin[s] / (W.ns * W.nr) * W.ns + o.kt) * W.nr;
+        // rows whose plane is within MERGE_XMAX of the extrapolation start (one row of margin; the exact
+        // test is below)
+        int r_lo = (int)floorf((float)(o.x2 - MERGE_XMAX - g.xtab[0]) / pitch) - 1;
+        int r_hi = (int)ceilf((float)(o.x2 + MERGE_XMAX - g.xtab[0]) / pitch) + 1;
+        r_lo = max(r_lo, 0);
+        r_hi = min(r_hi, W.nr - 1);
+        if (r_lo > r_hi) continue;
         unsigned long long best = ~0ull;
-        for (int k = 0; k < 2; k++) {
-            const int sgn = k == 0 ? +1 : -1;
-            const int kt = side0 + ((ks - side0) + (k == 0 ? 1 : half - 1)) % half;
-            if (k == 1 && kt == side0 + ((ks - side0) + 1) % half) break;   // tiny geometries
-            const long long X1 = p1.x, Y1 = p1.y, X2 = p2.x, Y2 = p2.y;
-            const long long x1 = (X1 * g.c30 + sgn * Y1 * g.s30) >> 30;
-            const long long y1 = (-sgn * X1 * g.s30 + Y1 * g.c30) >> 30;
-            const long long x2 = (X2 * g.c30 + sgn * Y2 * g.s30) >> 30;
-            const long long y2 = (-sgn * X2 * g.s30 + Y2 * g.c30) >> 30;
-            const long long dxs = x2 - x1;
-            if (dxs <= 0) continue;
-            // The extrapolated Y is monotonic in XT, so its range over the reach |XT - x2| <=
-            // MERGE_XMAX is that of the two ends.  If the window around it misses the range of the
-            // first-hit Y of every segment of sector kt, no T there can match (the usual case: S
-            // ends away from the edge that faces kt).
-            {
-                const long long ya = y1 + floor_div_pos((x2 - MERGE_XMAX - x1) * (y2 - y1), dxs);
-                const long long yb = y1 + floor_div_pos((x2 + MERGE_XMAX - x1) * (y2 - y1), dxs);
-                const long long ymin = ya < yb ? ya : yb, ymx = ya < yb ? yb : ya;
-                const long long bound = W.sec_ymax[ev * W.ns + kt];
-                if (ymin - W_MERGE > bound || ymx + W_MERGE < -bound) continue;
+        const float fy = (float)(o.y2 - o.y1) / (float)o.dxs, fz = (float)o.dz / (float)o.dxs;
+        const float y1 = (float)o.y1, z1 = (float)o.z1;
+        const int i1 = W.mrg_off[b0 + r_hi + 1];
+        for (int i = W.mrg_off[b0 + r_lo] + lane; i < i1; i += 32) {
+            const int4 e = merge_firsts(W)[i];
+            const long long XT = e.x;
+            const long long ax = XT - o.x2;
+            if ((ax < 0 ? -ax : ax) > MERGE_XMAX) continue;
+            {   // the windows in FP32, with margins above the floor and the rounding (a few 2^-24 of the
+                // terms): only pairs that the integer tests below reject are dropped
+                const float dx = (float)(XT - o.x1), py = dx * fy, pz = dx * fz;
+                if (fabsf((float)e.y - y1 - py) > (float)W_MERGE + 2.f + 1e-6f * (fabsf(y1) + fabsf(py)) ||
+                    fabsf((float)e.z - z1 - pz) > (float)W_MERGE + 2.f + 1e-6f * (fabsf(z1) + fabsf(pz)))
+                    continue;
             }
-            const int b0 = (ev * W.ns + kt) * W.nr;
-            // rows whose plane is within MERGE_XMAX of the extrapolation start (one row of margin;
-            // the exact test is below)
-            int r_lo = (int)floorf((float)(x2 - MERGE_XMAX - g.xtab[0]) / pitch) - 1;
-            int r_hi = (int)ceilf((float)(x2 + MERGE_XMAX - g.xtab[0]) / pitch) + 1;
-            r_lo = max(r_lo, 0);
-            r_hi = min(r_hi, W.nr - 1);
-            if (r_lo > r_hi) continue;
-            const int i1 = W.mrg_off[b0 + r_hi + 1];
-            for (int i = W.mrg_off[b0 + r_lo] + lane; i < i1; i += 32) {
-                const int t = W.mrg_list[i];
-                if (gap && W.prev[t] >= 0) continue;                 // a gap predecessor: no first segment
-                const int4 e = W.inend[t];
-                const long long XT = e.x;
-                const long long ax = XT - x2;
-                if ((ax < 0 ? -ax : ax) > MERGE_XMAX) continue;
-                const long long yp = y1 + floor_div_pos((XT - x1) * (y2 - y1), dxs);
-                const long long zp = p1.z + floor_div_pos((XT - x1) * (long long)(p2.z - p1.z), dxs);
-                const long long dy = e.y - yp, dz = e.z - zp;
-                if (dy > W_MERGE || dy < -W_MERGE || dz > W_MERGE || dz < -W_MERGE) continue;
-                const unsigned long long D = (unsigned long long)(dy * dy + dz * dz);
-                const unsigned long long kT = (D << 32) | (unsigned)t;
-                best = kT < best ? kT : best;
-                atomicMin(W.bestS + t, (D << 32) | (unsigned)s);
-            }
+            const int t = e.w;
+            if (gap && W.prev[t] >= 0) continue;                 // a gap predecessor: no first segment
+            const long long yp = o.y1 + floor_div_pos((XT - o.x1) * (o.y2 - o.y1), o.dxs);
+            const long long zp = o.z1 + floor_div_pos((XT - o.x1) * (long long)o.dz, o.dxs);
+            const long long dy = e.y - yp, dz = e.z - zp;
+            if (dy > W_MERGE || dy < -W_MERGE || dz > W_MERGE || dz < -W_MERGE) continue;
+            const unsigned long long D = (unsigned long long)(dy * dy + dz * dz);
+            const unsigned long long kT = (D << 32) | (unsigned)t;
+            best = kT < best ? kT : best;
+            atomicMin(W.bestS + t, (D << 32) | (unsigned)s);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, o);
+        for (int d = 16; d > 0; d >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, d);
             best = v < best ? v : best;
         }
-        if (lane == 0) W.bestT[s] = best;
+        if (lane == 0 && best != ~0ull) atomicMin(W.bestT + s, best);
     }
 }
 
@@ -450,7 +501,9 @@ void launch_merge(const Work &W, cudaStream_t s) {
         k_gap_match<<<grid, block, 0, s>>>(W);
         k_gap_link<<<grid, block, 0, s>>>(W);
     }
-    k_merge_match<<<grid, block, 0, s>>>(W);
+    // the list lives in the packed track hits, which are written below
+    k_merge_probe<<<W.sm_count * 8, 128, 0, s>>>(W, W.trk_pack);
+    k_merge_match<<<W.sm_count * 12, 128, 0, s>>>(W, W.trk_pack);
     k_merge_link<<<grid, block, 0, s>>>(W);
     k_merge_heads<<<grid, block, 0, s>>>(W);
     scan_exclusive(W.head, W.head_id, W.cap_chains, W.counters + CNT_NCHAINS, W.counters + CNT_NTRACKS,

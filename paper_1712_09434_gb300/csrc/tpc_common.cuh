@@ -146,6 +146,7 @@ enum {
     CNT_FRAME_H = 6,
     CNT_BINS_BAD = 7,         // set when the caller's bin offsets fail the check
     CNT_Q0 = 8,               // work-queue heads, one per kernel
+    CNT_MERGE = 26,           // outer ends listed for the sector merge
     CNT_STARTS = 25,          // chain starts listed
     CNT_ITS_PAIRS = 24,       // pairs left for the FP64 test of the ITS matching
     CNT_QFIT = 16,            // work-queue heads of the refit kernels under theta, by mode
