@@ -160,6 +160,10 @@ __global__ void __launch_bounds__(256) k_chain_write(Work W) {
     for (int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < W.nbins; b += nw) {
         const int c0 = W.bin_off[b], c1 = W.bin_off[b + 1];
         int pos = W.chain_off[b];
+        if (lane == 0) {      // the merge counts into these next
+            W.bin_cnt[b] = 0;
+            if (b % W.nr == 0) W.sec_ymax[b / W.nr] = 0;
+        }
         if (W.chain_off[b + 1] == pos) continue;
         for (int base = c0; base < c1; base += 32 * SWEEP) {
             int ln[SWEEP];

@@ -94,7 +94,7 @@ __global__ void k_merge_fill(Work W) {
             if (W.geom->xtab[mid] < e.x) lo = mid + 1; else hi = mid;
         }
         const int b = bin0 + lo;
-        const int p = W.mrg_off[b] + atomicAdd(W.bin_cnt + b, 1);
+        const int p = W.mrg_off[b] + atomicSub(W.bin_cnt + b, 1) - 1;
         W.mrg_list[p] = t;
         merge_firsts(W)[p] = make_int4(e.x, e.y, e.z, t);
     }
@@ -490,11 +490,9 @@ __global__ void k_event_offsets(Work W) {
 void launch_merge(const Work &W, cudaStream_t s) {
     const int block = W.tune.block[5] > 0 ? W.tune.block[5] : 128;
     const int grid = W.tune.grid[5] > 0 ? W.tune.grid[5] : W.sm_count * 8;
-    cudaMemsetAsync(W.bin_cnt, 0, sizeof(int32_t) * (W.nbins + 1), s);
-    cudaMemsetAsync(W.sec_ymax, 0, sizeof(int32_t) * (size_t)W.n_events * W.ns, s);
+    // bin_cnt and sec_ymax were reset by the chain stage
     k_merge_ends<<<grid, block, 0, s>>>(W);
     scan_exclusive(W.bin_cnt, W.mrg_off, W.nbins, nullptr, nullptr, W.scan_tmp, W.scan_tmp_len, s);
-    cudaMemsetAsync(W.bin_cnt, 0, sizeof(int32_t) * (W.nbins + 1), s);
     k_merge_fill<<<grid, block, 0, s>>>(W);
     if (W.rules & TPC_RULE_GAP_MERGE) {
         k_gap_back<<<grid, block, 0, s>>>(W);

@@ -707,8 +707,9 @@ __global__ void __launch_bounds__(LEN_BUCKETS) k_len_scan(int32_t *hist, int32_t
         sh[i] += v;
         __syncthreads();
     }
-    hist[i] = i > 0 ? sh[i - 1] : 0;          // exclusive offsets
-    hist[LEN_BUCKETS + i] = 0;               // fill counters
+    hist[i] = 0;                                            // counts of the next call
+    hist[LEN_BUCKETS + i] = i > 0 ? sh[i - 1] : 0;          // exclusive offsets
+    hist[2 * LEN_BUCKETS + i] = 0;                          // fill counters
     const int nch = (sh[LEN_BUCKETS - 1] + 31) / 32;
     // bucket of the first track of chunk c: the first one whose inclusive count exceeds 32 c
     auto bucket = [&](int c) {
@@ -755,9 +756,9 @@ __global__ void k_len_scatter(Work W, int32_t *hist, int32_t *order) {
         const unsigned peers = __match_any_sync(__activemask(), b);
         const int leader = __ffs(peers) - 1;
         int base = 0;
-        if (lane == leader) base = atomicAdd(hist + LEN_BUCKETS + b, __popc(peers));
+        if (lane == leader) base = atomicAdd(hist + 2 * LEN_BUCKETS + b, __popc(peers));
         base = __shfl_sync(peers, base, leader);
-        order[hist[b] + base + __popc(peers & ((1u << lane) - 1u))] = t;
+        order[hist[LEN_BUCKETS + b] + base + __popc(peers & ((1u << lane) - 1u))] = t;
     }
 }
 
@@ -815,7 +816,6 @@ int refit_part_doubles(int cap_tracks, int ns) { return ((cap_tracks + RED_T - 1
 void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
                       cudaStream_t s) {
     const CkLayout L = ck_layout(ck, ck_hits, ck_tracks);
-    cudaMemsetAsync(hist, 0, sizeof(int32_t) * LEN_BUCKETS, s);
     k_len_hist<<<W.sm_count * 4, 256, 0, s>>>(W, hist);
     k_len_scan<<<1, LEN_BUCKETS, 0, s>>>(hist, L.cb, L.cap_steps);
     k_len_scatter<<<W.sm_count * 4, 256, 0, s>>>(W, hist, order);

@@ -133,7 +133,7 @@ size_t layout(tpc_ctx *c, char *base) {
     carve(cur, c->rec, (size_t)refit_rec_words((int)C));
     carve(cur, c->part, (size_t)refit_part_doubles((int)C, c->hgeom.n_sectors));
     carve(cur, c->order, C + 1);
-    carve(cur, c->lhist, 1024);
+    carve(cur, c->lhist, 3 * 512);
     w.cap_chains = c->cap_chains;
     return (size_t)(cur - base);
 }
@@ -408,6 +408,7 @@ int tpc_reserve(tpc_ctx *c, int32_t max_clusters, int32_t max_events) {
     c->arena_bytes = bytes;
     layout(c, static_cast<char *>(p));
     TPC_CUDA(cudaMemset(c->ws.status, 0, 8 * sizeof(int32_t)));
+    TPC_CUDA(cudaMemset(c->lhist, 0, 3 * 512 * sizeof(int32_t)));
     return TPC_OK;
 }
 

@@ -210,7 +210,8 @@ void launch_select(const Work &W, cudaStream_t s);
 void launch_merge(const Work &W, cudaStream_t s);
 void launch_frame_merge(const Work &W, cudaStream_t s);
 // tracks in order of decreasing hit count into order, and the first step of every 32 of them in the
-// stored states of the gradient into its workspace ck (hist: 2 * 512 words of scratch)
+// stored states of the gradient into its workspace ck (hist: 3 * 512 words of scratch, whose
+// first 512 are 0 before and after)
 void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
                       cudaStream_t s);
 void launch_refit(const Work &W, const int32_t *order, cudaStream_t s);
