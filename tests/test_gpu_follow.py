@@ -1,12 +1,16 @@
 """The following against the oracle in both of its word sizes (the 32-bit filter needs ymax <= 16383
 and zmax <= 32767 LSB) at the ends of the coordinate ranges: drift length near 0 and near its
 maximum, times beyond the drift range (up to the last 16-bit value), the acceptance edge, steep
-slopes, with and without the skip-row rule."""
+slopes, with and without the skip-row rule; and in both mappings (eight lanes a task up to 2^20
+clusters of a call, a thread a task beyond), on these tracks and on the edge constructions."""
 import numpy as np
 import pytest
 
+import torch
+
 from oracle import oracle as O
 from paper_1712_09434_gb300 import capi
+from tests._constructed import edge_events
 
 pytestmark = pytest.mark.gpu
 
@@ -34,6 +38,52 @@ def _lines(rng, n, y_lo, y_hi, z_lo, z_hi, slope_z, drop, z_top):
     return p[:, 2].astype(np.int16), p[:, 3].astype(np.uint16), off
 
 
+def _noise(rng, ns, n):
+    """A second event without tracks, of n clusters spread over all rows."""
+    b = rng.integers(0, ns * NR, n)
+    p = np.unique(np.stack([b, rng.integers(-1300, 1300, n), rng.integers(0, 32000, n)], 1), axis=0)
+    off = np.searchsorted(p[:, 0], np.arange(ns * NR + 1)).astype(np.int32)
+    return p[:, 1].astype(np.int16), p[:, 2].astype(np.uint16), off
+
+
+def _check(pad, tim, off, ns, geo, og, rules, many):
+    """Candidates and tracks of the event against the oracle; many: with a noise event of 2^20 clusters
+    behind it."""
+    o = O.track_event(pad, tim, off, g=og, keep_stages=True, rules=rules)
+    nc, nt = len(o["cand_n"]), len(o["trk_off"]) - 1
+    assert nc > 10
+    n_ev = 1
+    if many:
+        q = _noise(np.random.default_rng(9), ns, (1 << 20) + 40000)
+        assert len(q[0]) > 1 << 20
+        off = np.concatenate([off[:-1], q[2] + off[-1]]).astype(np.int32)
+        pad, tim, n_ev = np.concatenate([pad, q[0]]), np.concatenate([tim, q[1]]), 2
+    cl = capi.Clusters.from_numpy(pad, tim, off, n_ev)
+    ctx = capi.Context(geometry=geo, max_clusters=cl.n_clusters, max_events=n_ev)
+    ctx.tpc_set_rules(rules)
+    tr = capi.Tracks(cl.n_clusters, n_ev, cl.n_clusters // 10 + 16, cl.n_clusters)
+    ctx.tpc_track_event(cl, tr)
+    assert ctx.tpc_sync_status() == 0
+
+    def get(what, n):
+        b = torch.empty(n, dtype=torch.int32, device="cuda")
+        ctx.tpc_debug_copy(what, b)
+        return b.cpu().numpy()
+
+    total = int(get(2, 1)[0])
+    assert total == nc or (many and total > nc)
+    np.testing.assert_array_equal(get(5, nc), o["cand_n"])
+    slots, rows = get(6, nc * NR).reshape(nc, NR), get(7, nc)
+    for t in range(nc):
+        s = slots[t, rows[t] & 0xffff:(rows[t] >> 16) + 1]
+        np.testing.assert_array_equal(s[s >= 0], o["cand_hits"][t][:o["cand_n"][t]])
+    g = tr.to_host()
+    assert g["ev_trk_off"][1] == nt
+    np.testing.assert_array_equal(g["trk_off"][:nt + 1], o["trk_off"])
+    np.testing.assert_array_equal(g["trk_hits"][:o["trk_off"][-1]], o["trk_hits"])
+    ctx.close()
+
+
 @pytest.mark.parametrize("lsb,zmax_cm", [(1.0 / 128, 250.0), (1.0 / 256, 250.0), (1.0 / 128, 255.9)])
 @pytest.mark.parametrize("rules", [0, 1])
 @pytest.mark.parametrize("y,z,slope_z", [
@@ -49,25 +99,12 @@ def test_following_words_match_the_oracle(lsb, zmax_cm, rules, y, z, slope_z):
     pad, tim, off = _lines(rng, 12, *y, *z, slope_z, 0.06 if rules else 0.02, 65535)
     geo = capi.tpc_geometry(NS, NR, 85.0, 247.0, 10.0, zmax_cm, lsb)
     og = O.geometry(n_sectors=NS, n_rows=NR, z_max=zmax_cm, lsb=lsb)
-    o = O.track_event(pad, tim, off, g=og, keep_stages=True, rules=rules)
-    cl = capi.Clusters.from_numpy(pad, tim, off, 1)
-    import torch
-    ctx = capi.Context(geometry=geo, max_clusters=cl.n_clusters, max_events=1)
-    ctx.tpc_set_rules(rules)
-    tr = capi.Tracks(cl.n_clusters, 1, cl.n_clusters // 10 + 16, cl.n_clusters)
-    ctx.tpc_track_event(cl, tr)
-    assert ctx.tpc_sync_status() == 0
-    nc = len(o["cand_n"])
-    assert nc > 20
-    get = lambda what, n: (lambda b: (ctx.tpc_debug_copy(what, b), b.cpu().numpy())[1])(
-        torch.empty(n, dtype=torch.int32, device="cuda"))
-    assert int(get(2, 1)[0]) == nc
-    np.testing.assert_array_equal(get(5, nc), o["cand_n"])
-    slots, rows = get(6, nc * NR).reshape(nc, NR), get(7, nc)
-    for t in range(nc):
-        s = slots[t, rows[t] & 0xffff:(rows[t] >> 16) + 1]
-        np.testing.assert_array_equal(s[s >= 0], o["cand_hits"][t][:o["cand_n"][t]])
-    g = tr.to_host()
-    np.testing.assert_array_equal(g["trk_off"], o["trk_off"])
-    np.testing.assert_array_equal(g["trk_hits"], o["trk_hits"])
-    ctx.close()
+    _check(pad, tim, off, NS, geo, og, rules, False)
+    if rules == 0:
+        _check(pad, tim, off, NS, geo, og, rules, True)
+
+
+@pytest.mark.parametrize("many", [False, True])
+def test_edge_events_in_both_mappings(many):
+    for pad, tim, off, _ in edge_events():
+        _check(pad, tim, off, 36, capi.default_geometry(), O.geometry(), 0, many)
