@@ -71,7 +71,7 @@ __global__ void k_merge_ends(Work W) {
         atomicMax(W.sec_ymax + W.chain_bin[t] / (W.ns * W.nr) * W.ns + sector, abs((int)W.pad[first]));
         atomicAdd(W.bin_cnt + (W.chain_bin[t] - W.chain_bin[t] % W.nr) + rf, 1);
         W.outend[2 * t] = make_int4(g.xtab[rB], W.pad[hB], W.tim[hB], sector);
-        W.outend[2 * t + 1] = make_int4(g.xtab[rL], W.pad[hL], W.tim[hL], 0);
+        W.outend[2 * t + 1] = make_int4(g.xtab[rL], W.pad[hL], W.tim[hL], rL);
     }
 }
 
@@ -128,75 +128,134 @@ __device__ __forceinline__ bool gap_inside(const DevGeom &g, const Abg &fy, cons
     return !((py < 0 ? -py : py) > g.ymax[row] || pz < 0 || pz > g.zmax || av > (long long)V_MAX * 65536);
 }
 
-// Backward filter of every accepted segment over its kept hits in descending rows: the state at its
-// first kept hit.  Also resets the gap keys.
-__global__ void k_gap_back(Work W) {
-    const int n = n_chains_of(W);
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        W.gap_bestT[t] = ~0ull;
-        W.gap_bestS[t] = ~0ull;
-        if (W.seg_n[t] < N_MIN) continue;
-        const Kept kept = kept_of(W, t);
-        const int32_t *sl = W.cand_slots + (size_t)t * W.nr;
-        Abg fy{}, fz{};
-        int k = 0, rprev = 0, h0 = -1;
-        for (int r = kept.r1; r >= kept.r0; r--) {
-            if (!kept.has(r)) continue;
-            const int h = sl[r];
-            if (k == 0) {
-                h0 = h;
-            } else if (k == 1) {
-                abg_init(fy, W.pad[h0], W.pad[h], rprev - r);
-                abg_init(fz, W.tim[h0], W.tim[h], rprev - r);
-                for (int j = rprev - r; j > 0; j--) { abg_predict(fy); abg_predict(fz); }
-                abg_update(fy, W.pad[h]);
-                abg_update(fz, W.tim[h]);
-            } else {
-                for (int j = rprev - r; j > 0; j--) { abg_predict(fy); abg_predict(fz); }
-                abg_update(fy, W.pad[h]);
-                abg_update(fz, W.tim[h]);
+// Calls f(row, y, z) for the kept hits of a segment in ascending (DIR +1) or descending rows; the
+// hits are loaded four at a time.
+template <int DIR, class F>
+__device__ __forceinline__ void kept_walk(const Work &W, const Kept &kept, const int32_t *sl, F f) {
+    const int last = (kept.r1 - kept.r0) >> 5;
+    int j = DIR > 0 ? 0 : last;
+    uint32_t m = kept.w[j];
+    for (;;) {
+        int row[4], h[4], y[4], z[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            while (!m && j + DIR >= 0 && j + DIR <= last) {
+                j += DIR;
+                m = kept.w[j];
             }
-            rprev = r;
-            k++;
+            row[q] = -1;
+            if (m) {
+                const int bit = DIR > 0 ? __ffs(m) - 1 : 31 - __clz(m);
+                row[q] = kept.r0 + 32 * j + bit;
+                m &= ~(1u << bit);
+            }
         }
-        long long *st = W.gap_state + 6 * (size_t)t;
-        st[0] = fy.p; st[1] = fy.v; st[2] = fy.a;
-        st[3] = fz.p; st[4] = fz.v; st[5] = fz.a;
+#pragma unroll
+        for (int q = 0; q < 4; q++) h[q] = row[q] >= 0 ? sl[row[q]] : 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            y[q] = row[q] >= 0 ? W.pad[h[q]] : 0;
+            z[q] = row[q] >= 0 ? W.tim[h[q]] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (row[q] >= 0) f(row[q], y[q], z[q]);
+        if (row[3] < 0) return;
     }
 }
 
-// Thread per segment S: forward filter over its kept hits, then row by row across the gap; every
-// segment T of the same sector whose first kept hit lies k >= M_MISS + 1 rows past S's last kept
-// hit is tested both ways; (D, T) kept for S, (D, S) offered to T by 64-bit atomicMin.
-__global__ void k_gap_match(Work W) {
-    const DevGeom &g = *W.geom;
-    const int n = n_chains_of(W);
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-        if (W.seg_n[s] < N_MIN) continue;
-        const Kept kept = kept_of(W, s);
-        const int32_t *sl = W.cand_slots + (size_t)s * W.nr;
-        Abg fy{}, fz{};
-        int k = 0, rprev = 0, h0 = -1, hl = -1;
-        for (int r = kept.r0; r <= kept.r1; r++) {
-            if (!kept.has(r)) continue;
-            const int h = sl[r];
-            if (k == 0) {
-                h0 = h;
-            } else {
-                if (k == 1) {
-                    abg_init(fy, W.pad[h0], W.pad[h], r - rprev);
-                    abg_init(fz, W.tim[h0], W.tim[h], r - rprev);
-                }
-                for (int j = r - rprev; j > 0; j--) { abg_predict(fy); abg_predict(fz); }
-                abg_update(fy, W.pad[h]);
-                abg_update(fz, W.tim[h]);
+// The filter over the kept hits of a segment in one direction; row, y0 and z0 are those of the last
+// hit taken.
+struct SegFilter {
+    Abg fy{}, fz{};
+    int k = 0, row = 0, y0 = 0, z0 = 0;
+    __device__ __forceinline__ void hit(int r, int y, int z) {
+        const int d = r > row ? r - row : row - r;
+        if (k > 0) {
+            if (k == 1) {
+                abg_init(fy, y0, y, d);
+                abg_init(fz, z0, z, d);
             }
-            rprev = r;
-            hl = h;
-            k++;
+            for (int j = d; j > 0; j--) {
+                abg_predict(fy);
+                abg_predict(fz);
+            }
+            abg_update(fy, y);
+            abg_update(fz, z);
         }
-        const int rs = rprev;
-        const long long ys = W.pad[hl], zs = W.tim[hl];
+        row = r;
+        y0 = y;
+        z0 = z;
+        k++;
+    }
+};
+
+// Accepted segments as a list in warp order (a fifth of the chains: the kernels below run with full
+// warps on it), and the reset of the gap keys.
+__global__ void __launch_bounds__(128) k_gap_list(Work W, int32_t *list) {
+    const int n = n_chains_of(W);
+    const int lane = threadIdx.x & 31;
+    for (int t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < n; t0 += gridDim.x * blockDim.x) {
+        const int t = t0 + lane;
+        bool acc = false;
+        if (t < n) {
+            W.gap_bestT[t] = ~0ull;
+            W.gap_bestS[t] = ~0ull;
+            acc = W.seg_n[t] >= N_MIN;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, acc);
+        int p = 0;
+        if (lane == 0 && m) p = atomicAdd(W.counters + CNT_GAP, __popc(m));
+        p = __shfl_sync(0xffffffffu, p, 0);
+        if (acc) list[p + __popc(m & ((1u << lane) - 1u))] = t;
+    }
+}
+
+// Forward filter state of a segment at its last kept hit: five words in the selection's claims (five
+// clusters or more per chain), the sixth in the 4-link successors; both are free by now.
+__device__ __forceinline__ long long *gap_fwd(const Work &W, int t, int k) {
+    return k < 5 ? reinterpret_cast<long long *>(W.claim) + 5 * (size_t)t + k
+                 : reinterpret_cast<long long *>(W.jump4) + t;
+}
+
+// Both filters of every accepted segment over its kept hits, a thread each: in descending rows to the
+// state at its first kept hit, and in ascending rows to the state at its last.
+__global__ void __launch_bounds__(128) k_gap_filter(Work W, const int32_t *list) {
+    const int n = W.counters[CNT_GAP];
+    const int n32 = (n + 31) & ~31;           // warps of one direction
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n32; i += gridDim.x * blockDim.x) {
+        const bool back = i < n32;
+        const int q = back ? i : i - n32;
+        if (q >= n) continue;
+        const int t = list[q];
+        const Kept kept = kept_of(W, t);
+        const int32_t *sl = W.cand_slots + (size_t)t * W.nr;
+        SegFilter f;
+        if (back) kept_walk<-1>(W, kept, sl, [&](int r, int y, int z) { f.hit(r, y, z); });
+        else kept_walk<1>(W, kept, sl, [&](int r, int y, int z) { f.hit(r, y, z); });
+        const long long st[6] = {f.fy.p, f.fy.v, f.fy.a, f.fz.p, f.fz.v, f.fz.a};
+#pragma unroll
+        for (int k = 0; k < 6; k++) *(back ? W.gap_state + 6 * (size_t)t + k : gap_fwd(W, t, k)) = st[k];
+    }
+}
+
+// Warp per segment S: its forward filter row by row across the gap; the lanes test the segments T of
+// the same sector whose first kept hit lies k >= M_MISS + 1 rows past S's last kept hit, both ways;
+// (D, T) kept for S, (D, S) offered to T by 64-bit atomicMin.  Behind a range of dead rows hundreds
+// of segments start in one row, and a thread per S took them one after the other: 79 + 333 us for
+// both filters and the tests of 147 k chains (28,991 tracks), now 5 + 74 + 134.
+__global__ void __launch_bounds__(128) k_gap_match(Work W, const int32_t *list) {
+    const DevGeom &g = *W.geom;
+    const int n = W.counters[CNT_GAP];
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int i0 = gw; i0 < n; i0 += nw) {
+        const int s = list[i0];
+        Abg fy{*gap_fwd(W, s, 0), *gap_fwd(W, s, 1), *gap_fwd(W, s, 2)};
+        Abg fz{*gap_fwd(W, s, 3), *gap_fwd(W, s, 4), *gap_fwd(W, s, 5)};
+        const int4 last = W.outend[2 * s + 1];
+        const int rs = last.w;
+        const long long ys = last.y, zs = last.z;
         const int b0 = W.chain_bin[s] - W.chain_bin[s] % W.nr;   // (event, sector) row 0
         unsigned long long best = ~0ull;
         for (int rt = rs + 1; rt < W.nr && rt <= rs + GAP_MAX; rt++) {
@@ -206,10 +265,11 @@ __global__ void k_gap_match(Work W) {
             if (rt - rs - 1 < M_MISS) continue;
             const long long py = q16_round(fy.p), pz = q16_round(fz.p);
             const long long w = W_F0 + (long long)W_F1 * (rt - rs - 1);
-            for (int i = W.mrg_off[b0 + rt]; i < W.mrg_off[b0 + rt + 1]; i++) {
-                const int t = W.mrg_list[i];
+            const int i1 = W.mrg_off[b0 + rt + 1];
+            for (int i = W.mrg_off[b0 + rt] + lane; i < i1; i += 32) {
+                const int4 e = merge_firsts(W)[i];
+                const int t = e.w;
                 if (t == s) continue;
-                const int4 e = W.inend[t];
                 const long long dy = e.y - py, dz = e.z - pz;
                 if (dy > w || dy < -w || dz > w || dz < -w || dy * dy + dz * dz > w * w) continue;
                 const long long *st = W.gap_state + 6 * (size_t)t;
@@ -229,7 +289,12 @@ __global__ void k_gap_match(Work W) {
                 atomicMin(W.gap_bestS + t, (D << 32) | (unsigned)s);
             }
         }
-        W.gap_bestT[s] = best;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, d);
+            best = v < best ? v : best;
+        }
+        if (lane == 0) W.gap_bestT[s] = best;
     }
 }
 
@@ -495,8 +560,10 @@ void launch_merge(const Work &W, cudaStream_t s) {
     scan_exclusive(W.bin_cnt, W.mrg_off, W.nbins, nullptr, nullptr, W.scan_tmp, W.scan_tmp_len, s);
     k_merge_fill<<<grid, block, 0, s>>>(W);
     if (W.rules & TPC_RULE_GAP_MERGE) {
-        k_gap_back<<<grid, block, 0, s>>>(W);
-        k_gap_match<<<grid, block, 0, s>>>(W);
+        // the list lives in the track heads, which are written below
+        k_gap_list<<<W.sm_count * 8, 128, 0, s>>>(W, W.trk_head);
+        k_gap_filter<<<W.sm_count * 10, 128, 0, s>>>(W, W.trk_head);
+        k_gap_match<<<W.sm_count * 14, 128, 0, s>>>(W, W.trk_head);
         k_gap_link<<<grid, block, 0, s>>>(W);
     }
     // the list lives in the packed track hits, which are written below

@@ -113,7 +113,7 @@ struct Work {
     int4 *inend;              // [cap_chains] first kept hit (Xtab, Y, Z, sector)
     int32_t *mrg_off;         // [nbins + 1] accepted segments per (event, sector, first row)
     int32_t *mrg_list;        // [cap_chains] segment indices in mrg_off order
-    int4 *outend;             // [cap_chains * 2] (X1, Y1, Z1, sector), (X2, Y2, Z2, -) of the outer end
+    int4 *outend;             // [cap_chains * 2] (X1, Y1, Z1, sector), (X2, Y2, Z2, row) of the outer end
     int32_t *sec_ymax;        // [max_events * n_sectors] largest |Y| of a segment's first kept hit
     int32_t *head;            // [cap_chains] 1 if the segment starts a merged track
     int32_t *head_id;         // [cap_chains + 1] exclusive scan of head = track id
@@ -146,6 +146,7 @@ enum {
     CNT_FRAME_H = 6,
     CNT_BINS_BAD = 7,         // set when the caller's bin offsets fail the check
     CNT_Q0 = 8,               // work-queue heads, one per kernel
+    CNT_GAP = 27,             // accepted segments listed for the gap merge
     CNT_MERGE = 26,           // outer ends listed for the sector merge
     CNT_STARTS = 25,          // chain starts listed
     CNT_ITS_PAIRS = 24,       // pairs left for the FP64 test of the ITS matching
