@@ -35,17 +35,17 @@ from paper_1712_09434_gb300 import synth  # noqa: E402
 
 METRIC = "TPC clusters/s tracked on 1 GB300, batched vs plain; adjoint calib-grad us/event"
 # kernels of one step (one graph): tracking (bin offset check 2, grid 1, links 1, chains 8, follow 2,
-# select 1, merge 17, length order of the tracks 3, refit 1) + refit and adjoint of its tracks
-# (forward and reverse pass 2, reduce 2; the stored-state form adds the chunk lengths and their
-# scan, 4; the hits were packed, the tracks sorted by length and the bin offsets checked by the
-# tracking part)
-LAUNCHES_TRACKING = 36
-LAUNCHES_REFIT_GRAD = {"checkpoints": 4, "stored states": 8}
+# select 1, merge 15, length order of the tracks 3, refit 1) + refit and adjoint of its tracks
+# (forward pass 1, reverse pass 2: stored states, and checkpoints for very long tracks; reduce 2; the
+# hits were packed, the tracks sorted by length and the bin offsets checked by the tracking part)
+LAUNCHES_TRACKING = 34
+LAUNCHES_REFIT_GRAD = {"checkpoints": 5, "stored states": 5}
 # copies of the central calibration event whose refit + adjoint run in one call (cost per event
 # when the gradient is summed over several events)
 CENTRAL_COPIES = 8
 
 def launches_per_step(tuning_best):
+    # the library stores the forward states whatever the shapes say; the shapes of a run name that form
     form = "stored states" if tuning_best and tuple(tuning_best.get("refit_grad", (0, 0, 0)))[2] == 1 else "checkpoints"
     return LAUNCHES_TRACKING + LAUNCHES_REFIT_GRAD[form], form
 WORKLOAD = "batch-64-events-logU-100-20000-tracks-20pct-noise"
@@ -639,8 +639,8 @@ def run_native(args, rank, world):
                 "loopers_with_both_legs_found": int(both.size),
                 "of_them_joined": float(np.isin(both, joined).mean()) if both.size else None}
     th5 = torch.tensor(synth.calib_theta(1005), dtype=torch.float64, device=dev)
-    # the adjoint as specified: per-row Kalman states recomputed in the reverse sweep from checkpoints
-    # (every 16 steps); then the variant that stores every step's input state (80 B per hit)
+    # the adjoint, with the library's default shapes and with the tuned form's (the same kernels since
+    # the library stores every step's input state, 80 B per hit, by default)
     from paper_1712_09434_gb300 import tune as _tune
     ms_grad, _ = timed(lambda: ctx.tpc_refit_grad(c5, t5, th5, s_chi2, grad, w5, a5, 1), 10, 3)
     g_ck = grad.clone()
@@ -751,7 +751,7 @@ def stage_bytes(u):
         "links": 18 * N,                # read own 4 B + neighbour-row grid 6 B; write up, down 8 B
         "chains": 16 * N + 12 * C,      # read up/down 8 B, write/read chain length 8 B; chain records
         "follow": 8 * Hc + 12 * C,      # candidate hit: slot write 4 B + cluster read 4 B; chain record
-        "select": 16 * Hc,              # candidate hit: slot read 4 B, claim 8 B, owner 4 B
+        "select": 16 * Hc,              # candidate hit: slot read 4 B, claim word 8 B, slot read again 4 B
         "merge": 12 * Ht + 32 * C,      # track hit: slot read + hit and label write; segment ends
         "refit": 8 * Ht + 92 * T,       # track hit: packed hit 8 B; per track 23 words out
         "pack": 16 * Ht,                # hit index 4 B + cluster 4 B in, packed hit 8 B out
@@ -815,16 +815,16 @@ def finish_native(args, res, world):
                     "event": "central, 20000 tracks, injected calibration, references at the vertex from the "
                              "TPC-ITS matching",
                     "tracks": res["n_tracks_c5"],
-                    "form": "refit + adjoint, Kalman states of the reverse sweep recomputed from checkpoints "
-                            "every 16 steps",
+                    "form": "refit + adjoint, the input state of every step stored (80 B per hit; checkpoints "
+                            "every 16 steps for tracks of 511 hits and more)",
                     "stored_states": {"value": res["ms_grad_event_stored"] * 1e3, "unit": "us/event",
-                                      "form": "variant storing every step's input state (80 B per hit); "
+                                      "form": "the same, timed a second time with the shapes that ask for it; "
                                               "identical gradient"},
                     "batched": {"value": res["ms_grad_copies"] * 1e3 / CENTRAL_COPIES, "unit": "us/event",
                                 "events": CENTRAL_COPIES,
                                 "stored_states": res["ms_grad_copies_stored"] * 1e3 / CENTRAL_COPIES,
                                 "form": "%d copies of the event tracked as one batch, refit + adjoint of all "
-                                        "their tracks in one call (checkpoints; stored_states: the variant); "
+                                        "their tracks in one call (stored_states: timed a second time); "
                                         "gradient checked to be %d times the event's" % (CENTRAL_COPIES,
                                                                                           CENTRAL_COPIES)}},
         "calibration": res["calib"],
