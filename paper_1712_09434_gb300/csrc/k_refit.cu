@@ -202,19 +202,36 @@ __device__ __forceinline__ int n_tracks_of(const Work &W) {
     return n < W.cap_tracks ? n : W.cap_tracks;
 }
 
+// Spread of few tracks over the chip: one thread in 2^spread takes a track, as long as the warps
+// are at most one a scheduler.  The lanes of a warp wait for each other's change of sector and
+// loads, so that fewer tracks a warp take fewer cycles a step: refit of a sector 136 -> 115 us, of a
+// full event 167 -> 161 us, objective of a full event 149 -> 139 us.  With up to two warps a
+// scheduler the objective takes 150 us again and with four 168 us.
+__device__ __forceinline__ int spread_of(const Work &W, int nt) {
+    const int room = W.sm_count * 128;   // a warp on each of the 4 schedulers
+    int sh = 0;
+    while (sh < 5 && ((long long)nt << (sh + 1)) <= room) sh++;
+    return sh;
+}
+
 // S8 at the nominal calibration: parameters, covariance, chi2, ndf of every track.
 // Tracks taken in the order of `order` (decreasing length) when given, so that the lanes of a warp
-// fit tracks of about the same length.  Eight blocks a multiprocessor cap it at 64 registers a
-// thread (a few spilled words): more resident warps hide the latency of the filter's FMA chain.
-// The offsets of S0 vanish here, so a hit needs no square root and division: 641 -> 557 us on 64
-// events (291,035 tracks), 239 -> 208 us on a central event, bit for bit the same parameters.  A
-// single event is bound by the latency of a track's steps (1.2 us each, about one warp a scheduler).
-__global__ void __launch_bounds__(128, 8) k_refit(Work W, const int32_t *order) {
+// fit tracks of about the same length.  MINB 8 caps it at 64 registers a thread (a few spilled
+// words): more resident warps hide the latency of the filter's FMA chain; MINB 5 (80 registers, none
+// spilled) is the better one where the tracks are resident at once anyway (208 -> 202 us on a
+// central event).  The offsets of S0 vanish here, so a hit needs no square root and division:
+// 641 -> 557 us on 64 events (291,035 tracks), 239 -> 208 us on a central event, bit for bit the same
+// parameters.  A single event is bound by the latency of a track's steps (about 1 us each).
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) k_refit(Work W, const int32_t *order) {
     const DevGeom &G = *W.geom;
     FitGeo fg;
     load_geo(G, fg);
     const int nt = n_tracks_of(W);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += gridDim.x * blockDim.x) {
+    const int sh = spread_of(W, nt);
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g >> sh < nt; g += gridDim.x * blockDim.x) {
+        if (g & ((1 << sh) - 1)) continue;
+        const int i = g >> sh;
         const int t = order ? order[i] : i;
         const int off = W.trk_off[t];
         int n = W.trk_off[t + 1] - off;
@@ -433,9 +450,15 @@ __global__ void __launch_bounds__(128, MINB) k_refit_grad(Work W, const double *
     if (MODE == 2 && L.cb[-1] == 0) return;
     __shared__ int s_item;
     int32_t *qh = W.counters + CNT_QFIT + MODE;
-    for (int base = queue_next(qh, blockDim.x, &s_item); base < nt; base = queue_next(qh, blockDim.x, &s_item)) {
-        const int i = base + threadIdx.x;
-        if (i >= nt) continue;
+    const int sh = MODE == 2 ? 0 : spread_of(W, nt), ng = nt << sh;
+    // At most one item a block: no queue, from which the first multiprocessors to start would take
+    // several and the others none (objective of a full event 239 -> 149 us, gradient of a central
+    // event: forward 296 -> 238, reverse 428 -> 385 us).
+    const bool once = ng <= (int)(gridDim.x * blockDim.x);
+    for (int base = once ? (int)(blockIdx.x * blockDim.x) : queue_next(qh, blockDim.x, &s_item); base < ng;
+         base = once ? ng : queue_next(qh, blockDim.x, &s_item)) {
+        const int i = (base + (int)threadIdx.x) >> sh;
+        if (i >= nt || (threadIdx.x & ((1 << sh) - 1))) continue;
         // first step of this chunk's stored states, or -1: the chunk keeps checkpoints
         const int cb = GRAD ? L.cb[i >> 5] : -1;
         if ((MODE == 2 && cb >= 0) || (MODE == 4 && cb < 0)) continue;
@@ -823,8 +846,11 @@ void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, l
 
 void launch_refit(const Work &W, const int32_t *order, cudaStream_t s) {
     const int block = W.tune.block[6] > 0 ? W.tune.block[6] : 128;
-    const int grid = W.tune.grid[6] > 0 ? W.tune.grid[6] : W.sm_count * 8;
-    k_refit<<<grid, block, 0, s>>>(W, order);
+    // one track a thread up to 311,000 tracks: 564 -> 530 us on 291,035 against half the blocks
+    const int grid = W.tune.grid[6] > 0 ? W.tune.grid[6] : W.sm_count * 16;
+    // about one track per 128 clusters, six blocks of 80 registers a multiprocessor
+    if (W.n_clusters / 128 <= 6 * 128 * W.sm_count) k_refit<5><<<grid, block, 0, s>>>(W, order);
+    else k_refit<8><<<grid, block, 0, s>>>(W, order);
 }
 
 void launch_refit_grad_fit(const Work &W, const double *theta, const float *weight, const float *anchor, int model,

@@ -77,3 +77,15 @@ def test_records_do_not_depend_on_how_states_are_kept(raw):
     many = _refit(ev, tracks, th, raw, pad_clusters=128 * 128 * 3 * sms + 128)[2]
     np.testing.assert_array_equal(many, base)
 
+
+
+@pytest.mark.parametrize("n", [608, 609, 1300, 4864, 9729, 155649])
+def test_records_do_not_depend_on_the_spread_over_warps(n):
+    # 152 x 128 threads are spread: 32 threads a track up to 608 tracks, one from 9,729 on; more
+    # tracks than threads are taken from the queue
+    ev, tracks = _tracks()
+    tracks = [t[-20:] for t in tracks]
+    th = _theta()
+    base = _refit(ev, tracks, th, True)[2]
+    many = _refit(ev, [tracks[i % len(tracks)] for i in range(n)], th, True)[2]
+    np.testing.assert_array_equal(many, base[np.arange(n) % len(tracks)])
