@@ -451,9 +451,9 @@ __global__ void __launch_bounds__(128, MINB) k_refit_grad(Work W, const double *
     __shared__ int s_item;
     int32_t *qh = W.counters + CNT_QFIT + MODE;
     const int sh = MODE == 2 ? 0 : spread_of(W, nt), ng = nt << sh;
-    // At most one item a block: no queue, from which the first multiprocessors to start would take
-    // several and the others none (objective of a full event 239 -> 149 us, gradient of a central
-    // event: forward 296 -> 238, reverse 428 -> 385 us).
+    // At most one item a block: no queue, which hands the items to whichever blocks reach it first
+    // (objective of a full event 239 -> 149 us, gradient of a central event: forward 296 -> 238,
+    // reverse 428 -> 385 us).
     const bool once = ng <= (int)(gridDim.x * blockDim.x);
     for (int base = once ? (int)(blockIdx.x * blockDim.x) : queue_next(qh, blockDim.x, &s_item); base < ng;
          base = once ? ng : queue_next(qh, blockDim.x, &s_item)) {
@@ -866,8 +866,8 @@ void launch_refit_grad_fit(const Work &W, const double *theta, const float *weig
         return;
     }
     // Reverse pass: where all tracks (about one per 128 clusters) are resident at once anyway, three
-    // blocks a multiprocessor without spilled registers are faster (central event 555 -> 432 us), else
-    // four (64 events 1579 -> 1455 us).  The register cap changes no bit of the result.
+    // blocks a multiprocessor without spilled registers are faster (central event 555 -> 386 us), else
+    // four (64 events 1579 -> 1440 us).  The register cap changes no bit of the result.
     k_refit_grad<3, 6><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
     if (W.n_clusters / 128 <= 3 * 128 * W.sm_count)
         k_refit_grad<4, 3><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
