@@ -492,9 +492,13 @@ __global__ void k_bins_check(const int32_t *in, int nbins, int n, int32_t *bad) 
     }
 }
 
-__global__ void k_bins_copy(const int32_t *in, int32_t *out, int nbins, int n, const int32_t *bad, int32_t *status) {
+// Also clears the counts of the length order (len_hist, if there is one).
+__global__ void k_bins_copy(const int32_t *in, int32_t *out, int nbins, int n, const int32_t *bad, int32_t *status,
+                            int32_t *len_hist) {
     const bool b = *bad != 0;
     if (b && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, ST_BOUNDS);
+    if (len_hist && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < LEN_BUCKETS; i += blockDim.x) len_hist[i] = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= nbins; i += gridDim.x * blockDim.x)
         out[i] = b ? (i == nbins ? n : 0) : in[i];
 }
@@ -505,7 +509,7 @@ void launch_bins_check(const Work &W, cudaStream_t s) {
     if (grid < 1) grid = 1;
     k_bins_check<<<grid, 256, 0, s>>>(W.bin_off_in, W.nbins, W.n_clusters, W.counters + CNT_BINS_BAD);
     k_bins_copy<<<grid, 256, 0, s>>>(W.bin_off_in, W.bin_ok, W.nbins, W.n_clusters, W.counters + CNT_BINS_BAD,
-                                     W.status);
+                                     W.status, W.len_hist);
 }
 
 void launch_grid(const Work &W, cudaStream_t s) {

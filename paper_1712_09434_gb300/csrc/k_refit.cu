@@ -22,7 +22,6 @@ namespace tpc {
 namespace {
 
 constexpr int CK_K = 16;           // steps between checkpoints
-constexpr int LEN_BUCKETS = 512;   // length classes of the length order; the last holds all longer tracks
 constexpr int ST_SLACK = 1024;     // spare steps per lane for the chunk padding of the stored states
 constexpr int CK_WORDS = 25;       // x, p[5], P lower triangle[15], frame, rref, yref, zref
 constexpr int ST_WORDS = 20;       // p[5], P lower triangle[15] (stored states: the rest from the hits)
@@ -730,7 +729,6 @@ __global__ void __launch_bounds__(LEN_BUCKETS) k_len_scan(int32_t *hist, int32_t
         sh[i] += v;
         __syncthreads();
     }
-    hist[i] = 0;                                            // counts of the next call
     hist[LEN_BUCKETS + i] = i > 0 ? sh[i - 1] : 0;          // exclusive offsets
     hist[2 * LEN_BUCKETS + i] = 0;                          // fill counters
     const int nch = (sh[LEN_BUCKETS - 1] + 31) / 32;
@@ -836,12 +834,12 @@ int refit_rec_words(int cap_tracks) { return cap_tracks * REC_WORDS; }
 int refit_part_doubles(int cap_tracks, int ns) { return ((cap_tracks + RED_T - 1) / RED_T + 1) * (2 * ns + 2); }
 
 
-void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
+void launch_len_order(const Work &W, int32_t *order, float *ck, long long ck_hits, long long ck_tracks,
                       cudaStream_t s) {
     const CkLayout L = ck_layout(ck, ck_hits, ck_tracks);
-    k_len_hist<<<W.sm_count * 4, 256, 0, s>>>(W, hist);
-    k_len_scan<<<1, LEN_BUCKETS, 0, s>>>(hist, L.cb, L.cap_steps);
-    k_len_scatter<<<W.sm_count * 4, 256, 0, s>>>(W, hist, order);
+    k_len_hist<<<W.sm_count * 4, 256, 0, s>>>(W, W.len_hist);
+    k_len_scan<<<1, LEN_BUCKETS, 0, s>>>(W.len_hist, L.cb, L.cap_steps);
+    k_len_scatter<<<W.sm_count * 4, 256, 0, s>>>(W, W.len_hist, order);
 }
 
 void launch_refit(const Work &W, const int32_t *order, cudaStream_t s) {
@@ -855,12 +853,12 @@ void launch_refit(const Work &W, const int32_t *order, cudaStream_t s) {
 
 void launch_refit_grad_fit(const Work &W, const double *theta, const float *weight, const float *anchor, int model,
                            bool grad, float *ck, long long ck_hits, long long ck_tracks, float *rec, int32_t *order,
-                           int32_t *hist, bool sorted, cudaStream_t s) {
+                           bool sorted, cudaStream_t s) {
     const int block = W.tune.block[7] > 0 ? W.tune.block[7] : 128;
     const int grid = W.tune.grid[7] > 0 ? W.tune.grid[7] : W.sm_count * 8;
     const CkLayout L = ck_layout(ck, ck_hits, ck_tracks);
     cudaMemsetAsync(W.counters + CNT_QFIT, 0, 5 * sizeof(int32_t), s);
-    if (!sorted) launch_len_order(W, order, hist, ck, ck_hits, ck_tracks, s);
+    if (!sorted) launch_len_order(W, order, ck, ck_hits, ck_tracks, s);
     if (!grad) {
         k_refit_grad<0, 1><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
         return;

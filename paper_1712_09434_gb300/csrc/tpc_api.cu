@@ -24,7 +24,7 @@ struct tpc_ctx {
     Work ws;                  // workspace part of the kernel arguments
     float *ck, *rec;
     double *part;
-    int32_t *order, *lhist;   // tracks by decreasing length for the adjoint
+    int32_t *order;           // tracks by decreasing length for the refit and the adjoint
     // batch graph cache
     cudaStream_t cap_stream;
     // a few graphs, keyed by the kernel arguments (e.g. double-buffered inputs), least recently
@@ -133,7 +133,7 @@ size_t layout(tpc_ctx *c, char *base) {
     carve(cur, c->rec, (size_t)refit_rec_words((int)C));
     carve(cur, c->part, (size_t)refit_part_doubles((int)C, c->hgeom.n_sectors));
     carve(cur, c->order, C + 1);
-    carve(cur, c->lhist, 3 * 512);
+    carve(cur, w.len_hist, 3 * LEN_BUCKETS);
     w.cap_chains = c->cap_chains;
     return (size_t)(cur - base);
 }
@@ -218,7 +218,7 @@ int enqueue_pipeline(const tpc_ctx *c, const Work &W, cudaStream_t s, bool captu
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[5], s, evf));
     launch_merge(W, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[6], s, evf));
-    launch_len_order(W, c->order, c->lhist, c->ck, (long long)c->max_clusters + 1, (long long)c->cap_chains + 1, s);
+    launch_len_order(W, c->order, c->ck, (long long)c->max_clusters + 1, (long long)c->cap_chains + 1, s);
     launch_refit(W, c->order, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_pipe[7], s, evf));
     return cuda_err(cudaGetLastError());
@@ -252,7 +252,7 @@ int enqueue_refit_grad(const tpc_ctx *c, const Work &W, const int32_t *n_tracks_
     }
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_refit[1], s, evf));
     launch_refit_grad_fit(W, theta, weight, anchor, model, grad != nullptr, c->ck, (long long)c->max_clusters + 1,
-                          (long long)c->cap_chains + 1, c->rec, c->order, c->lhist, !pack, s);
+                          (long long)c->cap_chains + 1, c->rec, c->order, !pack, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_refit[2], s, evf));
     launch_refit_grad_reduce(W, sum_chi2, grad, c->rec, c->part, s);
     if (prof) TPC_CUDA(cudaEventRecordWithFlags(c->ev_refit[3], s, evf));
@@ -408,7 +408,6 @@ int tpc_reserve(tpc_ctx *c, int32_t max_clusters, int32_t max_events) {
     c->arena_bytes = bytes;
     layout(c, static_cast<char *>(p));
     TPC_CUDA(cudaMemset(c->ws.status, 0, 8 * sizeof(int32_t)));
-    TPC_CUDA(cudaMemset(c->lhist, 0, 3 * 512 * sizeof(int32_t)));
     return TPC_OK;
 }
 

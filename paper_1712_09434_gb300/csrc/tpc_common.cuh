@@ -30,6 +30,7 @@ constexpr int MAX_SECTORS = 64;
 constexpr int ZB_SHIFT = 9;       // grid Z slab = 512 LSB (4 cm): a +-384 window spans <= 2 slabs
 constexpr int NZB = 64;           // slabs per row bin (Z >> 9 clamped to 63)
 constexpr int ZOFF_STRIDE = NZB + 1;
+constexpr int LEN_BUCKETS = 512;  // length classes of the length order; the last holds all longer tracks
 
 constexpr float SIGMA2 = 0.01f;   // measurement variance (cm^2)
 constexpr float SNP_MAX = 0.999f; // |sin phi| limit of the local helix state
@@ -126,6 +127,9 @@ struct Work {
     // time-frame slice merge (S11): the per-slice tracks it reads (device)
     const int32_t *s_trk_off, *s_trk_hits, *s_ev_trk_off, *s_n_tracks;
     int slice_len;
+    // length order of the tracks: counts, offsets and fill levels of the classes.  The counts are
+    // cleared by the check of the bin offsets, which every call that sorts makes first on its stream
+    int32_t *len_hist;        // [3 * LEN_BUCKETS] (nullptr: a call without a workspace)
     // scan scratch
     int32_t *scan_tmp;        // [scan_tmp_len]
     int scan_tmp_len;
@@ -211,15 +215,14 @@ void launch_select(const Work &W, cudaStream_t s);
 void launch_merge(const Work &W, cudaStream_t s);
 void launch_frame_merge(const Work &W, cudaStream_t s);
 // tracks in order of decreasing hit count into order, and the first step of every 32 of them in the
-// stored states of the gradient into its workspace ck (hist: 3 * 512 words of scratch, whose
-// first 512 are 0 before and after)
-void launch_len_order(const Work &W, int32_t *order, int32_t *hist, float *ck, long long ck_hits, long long ck_tracks,
+// stored states of the gradient into its workspace ck; launch_bins_check comes before it on s
+void launch_len_order(const Work &W, int32_t *order, float *ck, long long ck_hits, long long ck_tracks,
                       cudaStream_t s);
 void launch_refit(const Work &W, const int32_t *order, cudaStream_t s);
 // sorted: order already holds the length order of these tracks
 void launch_refit_grad_fit(const Work &W, const double *theta, const float *weight, const float *anchor, int model,
                            bool grad, float *ck, long long ck_hits, long long ck_tracks, float *rec, int32_t *order,
-                           int32_t *hist, bool sorted, cudaStream_t s);
+                           bool sorted, cudaStream_t s);
 void launch_refit_grad_reduce(const Work &W, double *sum_chi2, double *grad, const float *rec, double *part,
                               cudaStream_t s);
 size_t refit_ck_words(long long cap_hits, long long cap_tracks);
