@@ -407,7 +407,9 @@ int tpc_reserve(tpc_ctx *c, int32_t max_clusters, int32_t max_events) {
     c->arena = p;
     c->arena_bytes = bytes;
     layout(c, static_cast<char *>(p));
-    TPC_CUDA(cudaMemset(c->ws.status, 0, 8 * sizeof(int32_t)));
+    // cleared before the first call can run, whatever its stream and whatever the default stream holds
+    TPC_CUDA(cudaMemsetAsync(c->ws.status, 0, 8 * sizeof(int32_t), c->cap_stream));
+    TPC_CUDA(cudaStreamSynchronize(c->cap_stream));
     return TPC_OK;
 }
 
@@ -624,10 +626,10 @@ int tpc_rule_constants(int64_t *out, int32_t cap) {
 int tpc_sync_status(tpc_ctx *c, void *stream) {
     if (!c || !c->arena) return TPC_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    TPC_CUDA(cudaStreamSynchronize(s));
     int32_t st = 0;
-    TPC_CUDA(cudaMemcpy(&st, c->ws.status, sizeof(st), cudaMemcpyDeviceToHost));
-    TPC_CUDA(cudaMemset(c->ws.status, 0, sizeof(int32_t)));
+    TPC_CUDA(cudaMemcpyAsync(&st, c->ws.status, sizeof(st), cudaMemcpyDeviceToHost, s));
+    TPC_CUDA(cudaMemsetAsync(c->ws.status, 0, sizeof(int32_t), s));
+    TPC_CUDA(cudaStreamSynchronize(s));
     if (st & ST_TIMEOUT) return TPC_ERR_TIMEOUT;
     if (st & ST_BOUNDS) return TPC_ERR_BOUNDS;
     if (st & ST_CAPACITY) return TPC_ERR_CAPACITY;

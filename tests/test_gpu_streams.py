@@ -66,3 +66,25 @@ def test_first_call_of_a_workspace_on_a_stream_that_does_not_wait(grown):
     np.testing.assert_array_equal(ref[2].cpu().numpy(), got[2].cpu().numpy())
     ctx.close()
     del busy
+
+
+def test_an_error_on_a_stream_that_does_not_wait_is_not_lost():
+    ev = synth.make_event(synth.full_event(seed=31, n_tracks=300))
+    off = ev.bin_off.copy()
+    off[-1] -= 1                       # the offsets do not end at the number of clusters
+    cl = capi.Clusters.from_numpy(ev.pad_fp, ev.time_fp, off, 1)
+    tr = _outputs(ev)[0]
+    warm = _gpu.make_context(ev.n_clusters, 1)         # kernels loaded: loading them waits for the device
+    warm.tpc_track_event(_gpu.clusters_of(ev), tr)
+    assert warm.tpc_sync_status() == 0
+    ctx = capi.Context()
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    busy = _queue_work()
+    ctx.reserve(ev.n_clusters, 1)
+    ctx.tpc_track_event(cl, tr, stream=side)
+    assert ctx.tpc_sync_status(stream=side) == capi.TPC_ERR_BOUNDS
+    assert ctx.tpc_sync_status(stream=side) == capi.TPC_OK       # read and cleared
+    torch.cuda.synchronize()
+    ctx.close()
+    del busy
