@@ -439,6 +439,7 @@ __global__ void __launch_bounds__(128, MINB) k_refit_grad(Work W, const double *
     float *ck = L.ck;
     constexpr bool GRAD = MODE != 0;
     __shared__ float th[NPAR_MAX];
+    if (MODE == 2 && L.cb[-1] == 0) return;      // no chunk keeps checkpoints
     const DevGeom &G = *W.geom;
     const int ns = W.ns, np = 1 + 2 * ns;
     for (int i = threadIdx.x; i < np; i += blockDim.x) th[i] = (float)(i == 0 ? 1.0 - theta[0] : theta[i]);
@@ -446,10 +447,9 @@ __global__ void __launch_bounds__(128, MINB) k_refit_grad(Work W, const double *
     FitGeo fg;
     load_geo(G, fg);
     const int nt = n_tracks_of(W);
-    if (MODE == 2 && L.cb[-1] == 0) return;
     __shared__ int s_item;
     int32_t *qh = W.counters + CNT_QFIT + MODE;
-    const int sh = MODE == 2 ? 0 : spread_of(W, nt), ng = nt << sh;
+    const int sh = spread_of(W, nt), ng = nt << sh;
     // At most one item a block: no queue, which hands the items to whichever blocks reach it first
     // (objective of a full event 239 -> 149 us, gradient of a central event: forward 296 -> 238,
     // reverse 428 -> 385 us).
@@ -871,7 +871,10 @@ void launch_refit_grad_fit(const Work &W, const double *theta, const float *weig
         k_refit_grad<4, 3><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
     else
         k_refit_grad<4, 4><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
-    k_refit_grad<2, 4><<<W.sm_count, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
+    // Tracks with checkpoints: as many blocks as the other passes, and spread like theirs (reverse pass of
+    // 20 / 2,000 / 25,000 / 60,000 tracks of 520 hits and more 2.07 / 3.6 / 7.8 / 9.3 ms; one block a
+    // multiprocessor without spread 3.3 / 6.3 / 11.1 / 19.9).  Without such tracks it takes 2.2 us.
+    k_refit_grad<2, 4><<<grid, block, 0, s>>>(W, theta, weight, anchor, model, L, rec, order);
 }
 
 void launch_refit_grad_reduce(const Work &W, double *sum_chi2, double *grad, const float *rec, double *part,
