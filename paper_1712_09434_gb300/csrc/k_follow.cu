@@ -1,14 +1,15 @@
-// S5 track following: Kalman-filter following of each seed across the pad rows, one thread per
-// track candidate (arxiv 1712.09434 section 3).  Every accept/reject decision is taken by an
-// integer steady-state Kalman filter (alpha-beta-gamma = 1/2, 1/8, 1/32 on a Q16 state, floor
-// shifts, int64) so that the hit lists are bit-identical to an independent FP64 implementation;
-// the floating-point Kalman filter is used for the parameters only (S8).
+// S5 track following: Kalman-filter following of each seed across the pad rows (arxiv 1712.09434
+// section 3).  Every accept/reject decision is taken by an integer steady-state Kalman filter (abg.cuh:
+// alpha-beta-gamma = 1/2, 1/8, 1/32 on a Q16 state, floor shifts) so that the hit lists are
+// bit-identical to an independent FP64 implementation; the floating-point Kalman filter is used for
+// the parameters only (S8).
 //
 // A chain is followed by two threads at once: one filters along it in ascending rows and extends it
-// row by row outwards, the other filters in descending rows and extends it inwards.  A step: predict, look up the nearest cluster (minimum (d^2, index)) within a
-// radius that grows with consecutive misses in the row's Z-slab grid, update.  A candidate is
-// stored as one cluster per row (-1 for a miss) between its first and last row.  The chains are
-// taken in an order that groups chains of equal length and nearby start rows in a warp (below).
+// row by row outwards, the other filters in descending rows and extends it inwards.  A step: predict,
+// look up the nearest cluster (minimum (d^2, index)) within a radius that grows with consecutive
+// misses in the row's Z-slab grid, update.  A candidate is stored as one cluster per row (-1 for a
+// miss) between its first and last row.  The chains are taken in an order that groups chains of equal
+// length and nearby start rows in a warp (below).
 //
 // What bounds it: the dependent loads of one thread's steps (link, coordinates; slab offsets, search)
 // and the instructions of a divergent search, over the threads in flight.  Two threads a chain halve
@@ -19,52 +20,13 @@
 // 5,000-track event 446 -> 360 us, one sector of 138 chains 350 -> 190 us; with the 64-bit filter
 // 3.79 ms, 746, 331 and 213 us.  Reading a slab four entries at a time instead of by binary search
 // was slower where rows are dense (4.0 ms, 802 us).
+#include "abg.cuh"
 #include "tpc_common.cuh"
 
 namespace tpc {
 
 namespace {
 
-// The filter word T is int64, or int32 for geometries with ymax <= 16383 and zmax <= 32767 (narrow):
-// then a Q16 coordinate fits 32 bits, with Z shifted by -16384 so that one step never carries a
-// prediction past the word (a step moves less than 16384 LSB: the velocity that a track can build
-// up inside the drift range at 343 LSB per residual stays below that).  Sums and differences are
-// exact modulo 2^32 in any case, so only the reading of a prediction could be wrong, for a hit more
-// than 16384 LSB beyond the drift range; such a chain is not extended (it would stop at once).
-template <class T>
-struct Abg {
-    static constexpr int ZB = sizeof(T) == 4 ? 16384 : 0;   // Z as the filter holds it: z - ZB
-    T p, v, a;
-};
-template <class T>
-__device__ __forceinline__ T q16(int m) {
-    if constexpr (sizeof(T) == 4) return (T)((uint32_t)m << 16);
-    else return (T)m * 65536;
-}
-
-// state at m0 with the velocity of the step to m1, drow = 1 or 2 rows further (2 across a row that
-// a link skips; the division is exact)
-template <class T>
-__device__ __forceinline__ void abg_init(Abg<T> &f, int m0, int m1, int drow) {
-    f.p = q16<T>(m0);
-    f.v = (T)(m1 - m0) * (65536 / drow);
-    f.a = 0;
-}
-template <class T>
-__device__ __forceinline__ void abg_predict(Abg<T> &f) {
-    f.p += f.v + (f.a >> 1);
-    f.v += f.a;
-}
-template <class T>
-__device__ __forceinline__ void abg_update(Abg<T> &f, int m) {
-    const T e = q16<T>(m) - f.p;
-    f.p += e >> 1;
-    f.v += e >> 3;
-    f.a += e >> 5;
-}
-template <class T>
-__device__ __forceinline__ int q16_round(T p) { return (int)((p + 32768) >> 16); }
-constexpr int NARROW_YMAX = 16383, NARROW_ZMAX = 32767, NARROW_ZHIT = 49151;
 __device__ __forceinline__ int slab_of(int z) { int s = z >> ZB_SHIFT; return s < NZB - 1 ? s : NZB - 1; }
 
 // Nearest cluster of a row (its grid entries yz, indices loc, slab offsets zo) to (py, pz) with
@@ -363,7 +325,7 @@ __global__ void __launch_bounds__(FG_BLOCK) k_follow_few(Work W, const int32_t *
             c_next = __ldg(W.bin_off + rowbase + r);
             zo = __ldg(W.zoff + (size_t)(rowbase + r) * ZOFF_STRIDE + min(zs + j, NZB));
         };
-        if (act) ahead(row, q16_round(f.fz.p + f.fz.v + (f.fz.a >> 1)) + A::ZB);
+        if (act) ahead(row, q16_round(abg_ahead(f.fz)) + A::ZB);
         while (__any_sync(FULL, act)) {
             const int c0 = c_next, zs0 = zs, zo0 = zo;
             int py = 0, pz = 0, w = 0;
