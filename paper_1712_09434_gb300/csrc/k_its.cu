@@ -211,6 +211,9 @@ __global__ void __launch_bounds__(128) k_its_scan(Work W, ItsArgs A) {
         const float m0_32 = (float)(q[5] + ITS_SIGMA_Y * ITS_SIGMA_Y), pss32 = (float)q[7];
         const float ptt32 = (float)q[10], pqq32 = (float)q[14];
         const float g = (float)ITS_CHI2 * 1.001f;
+        const float mtl = 1e-3f + 1e-6f * fabsf(tl32), mz = 1e-3f + 1e-6f * fabsf(z32);
+        const float m2 = 1e-6f * (1.f + fabsf(tl32)), m3 = 1e-6f * (1.f + fabsf(q32));
+        auto beyond = [](float d, float m) { return fmaxf(fabsf(d) - m, 0.f); };     // (NaN: 0, left to FP64)
         if (d0_32 * d0_32 > g * m0_32) continue;
         const int b0 = (int)floor((phi_t - ITS_DPHI) / TWO_PI * ITS_NPHI), b1 = (int)floor((phi_t + ITS_DPHI) / TWO_PI * ITS_NPHI);
         // the tan lambda bins that can hold an ITS track within the window (and its margin)
@@ -219,16 +222,18 @@ __global__ void __launch_bounds__(128) k_its_scan(Work W, ItsArgs A) {
             const int bp = ((bb % ITS_NPHI) + ITS_NPHI) % ITS_NPHI;
             const int j1 = A.off[bp * ITS_NTL + tb1];
             for (int j = A.off[bp * ITS_NTL + tb0] + sub; j < j1; j += ITS_LANES) {
-                // FP32 pre-checks with margins far above FP32 rounding (1e-3 in tan lambda and z, 1e-3
-                // rad, 0.1 % of the one-component chi2 bound): they only reject pairs that the FP64
-                // tests reject too
+                // FP32 pre-checks that only reject pairs that the FP64 tests reject too: the margins lie far
+                // above FP32 rounding, which is relative to the operands (1e-3 and 1e-6 of the value in
+                // tan lambda, z and azimuth; 1e-6 and 1e-6 of the value of a component's distance, which
+                // the caller's errors may fall below, and 0.1 % of the one-component chi2 bound)
                 const float4 r = A.srt[3 * (size_t)j], e = A.srt[3 * (size_t)j + 1], sc = A.srt[3 * (size_t)j + 2];
-                if (fabsf(r.z - tl32) > (float)ITS_DTL + 1e-3f || fabsf(r.y - z32) > (float)ITS_DZ + 1e-3f) continue;
+                if (fabsf(r.z - tl32) > (float)ITS_DTL + mtl || fabsf(r.y - z32) > (float)ITS_DZ + mz) continue;
                 float dph = r.x - phi32;
                 dph -= rintf(dph * (float)(1.0 / TWO_PI)) * (float)TWO_PI;
-                if (fabsf(dph) > (float)ITS_DPHI + 1e-3f) continue;
-                const float sdp = sc.x * ca32 - sc.y * sa32, cph = (sc.y * ca32 + sc.x * sa32) * e.x;
-                const float d1 = sn32 - sdp, d2 = tl32 - r.z, d3 = q32 - r.w;
+                if (fabsf(dph) > (float)ITS_DPHI + 1e-3f + 1e-6f * fabsf(r.x)) continue;
+                // distances taken smaller, the error in sin phi larger than they are by the rounding
+                const float sdp = sc.x * ca32 - sc.y * sa32, cph = (fabsf(sc.y * ca32 + sc.x * sa32) + 1e-6f) * e.x;
+                const float d1 = beyond(sn32 - sdp, 2e-6f), d2 = beyond(tl32 - r.z, m2), d3 = beyond(q32 - r.w, m3);
                 if (d1 * d1 > g * (pss32 + cph * cph) || d2 * d2 > g * (ptt32 + e.y * e.y) ||
                     d3 * d3 > g * (pqq32 + e.z * e.z))
                     continue;
