@@ -33,13 +33,15 @@ __device__ __forceinline__ uint32_t key_of(int n_rows, int n_hits, int local) {
     return ((uint32_t)(n_rows - n_hits) << 23) | (uint32_t)local;
 }
 
-// Barrier of the blocks that share an item: release / acquire at the scope of the group.
+// Barrier of the blocks that share an item: release / acquire at the scope of the group.  Every thread
+// arrives on its own (no .aligned): the loops before it end at different times for the lanes of a
+// warp, and nothing but the compiler would bring them together again.
 template <int CS>
 __device__ __forceinline__ void group_sync() {
     if constexpr (CS == 1) {
         __syncthreads();
     } else {
-        asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
     }
 }
 
