@@ -40,14 +40,21 @@ METRIC = "TPC clusters/s tracked on 1 GB300, batched vs plain; adjoint calib-gra
 # hits were packed, the tracks sorted by length and the bin offsets checked by the tracking part)
 LAUNCHES_TRACKING = 34
 LAUNCHES_REFIT_GRAD = {"checkpoints": 5, "stored states": 5}
+ADJOINT_FORM = "stored states"    # what the library runs, whatever the launch shapes say
 # copies of the central calibration event whose refit + adjoint run in one call (cost per event
 # when the gradient is summed over several events)
 CENTRAL_COPIES = 8
 
-def launches_per_step(tuning_best):
-    # the library stores the forward states whatever the shapes say; the shapes of a run name that form
-    form = "stored states" if tuning_best and tuple(tuning_best.get("refit_grad", (0, 0, 0)))[2] == 1 else "checkpoints"
-    return LAUNCHES_TRACKING + LAUNCHES_REFIT_GRAD[form], form
+
+def adjoint_form(res):
+    """The form of the gradient in a result: named by every run of this file.  One that does not name
+    it is of a library where the launch shapes chose (checkpoints unless the chunk was 1)."""
+    if "adjoint_form" in res:
+        return res["adjoint_form"]
+    best = res["tuning"].get("best")
+    return "stored states" if best and tuple(best.get("refit_grad", (0, 0, 0)))[2] == 1 else "checkpoints"
+
+
 WORKLOAD = "batch-64-events-logU-100-20000-tracks-20pct-noise"
 
 
@@ -364,7 +371,7 @@ def run_native(args, rank, world):
 
     out = {"ms_step": ms_all, "ms_single": ms_single, "n_clusters": n_clusters, "n_clusters_all": n_cl_all,
            "n_tracks": n_tracks,
-           "n_hits": n_hits, "clocks": clk, "tuning": tuning_info, "prof": prof}
+           "n_hits": n_hits, "clocks": clk, "tuning": tuning_info, "prof": prof, "adjoint_form": ADJOINT_FORM}
     if args.only_step:
         return out
     # the measured FP32 roof of the Kalman stages (seconds-long FMA loop, clocks sampled)
@@ -639,15 +646,9 @@ def run_native(args, rank, world):
                 "loopers_with_both_legs_found": int(both.size),
                 "of_them_joined": float(np.isin(both, joined).mean()) if both.size else None}
     th5 = torch.tensor(synth.calib_theta(1005), dtype=torch.float64, device=dev)
-    # the adjoint, with the library's default shapes and with the tuned form's (the same kernels since
-    # the library stores every step's input state, 80 B per hit, by default)
-    from paper_1712_09434_gb300 import tune as _tune
+    # the adjoint, with the library's default shapes
     ms_grad, _ = timed(lambda: ctx.tpc_refit_grad(c5, t5, th5, s_chi2, grad, w5, a5, 1), 10, 3)
-    g_ck = grad.clone()
-    ctx.tpc_set_tuning(_tune.to_struct({"refit_grad": (0, 0, 1)}))
-    ms_grad_stored, _ = timed(lambda: ctx.tpc_refit_grad(c5, t5, th5, s_chi2, grad, w5, a5, 1), 10, 3)
-    ctx.tpc_set_tuning(None)
-    assert torch.equal(g_ck, grad), "the two adjoint forms must give identical gradients"
+    g_ev = grad.clone()
     # the same refit + adjoint over K copies of the event tracked as one batch, in one call: the
     # cost per event when the calibration sums its gradient over several events (one event alone
     # fills about one warp per SM sub-partition, so its time is the latency of its longest tracks)
@@ -663,11 +664,8 @@ def run_native(args, rank, world):
     wK, aK = w5.repeat(K), a5.repeat(K, 1)
     gK = torch.empty_like(grad)
     ms_grad_K, _ = timed(lambda: ctx.tpc_refit_grad(cK, tK, th5, s_chi2, gK, wK, aK, 1), 10, 3)
-    assert torch.allclose(gK, K * g_ck, rtol=1e-9, atol=1e-9 * float(g_ck.abs().max())), \
+    assert torch.allclose(gK, K * g_ev, rtol=1e-9, atol=1e-9 * float(g_ev.abs().max())), \
         "K copies must give K times the event's gradient"
-    ctx.tpc_set_tuning(_tune.to_struct({"refit_grad": (0, 0, 1)}))
-    ms_grad_K_stored, _ = timed(lambda: ctx.tpc_refit_grad(cK, tK, th5, s_chi2, gK, wK, aK, 1), 10, 3)
-    ctx.tpc_set_tuning(None)
     del cK, tK, bK
 
     # plain per-event tracking of single events: the central event above and a 5,000-track event
@@ -715,8 +713,7 @@ def run_native(args, rank, world):
                  "sum_chi2_start_end": [cres.history[0][1], cres.history[-1][1]],
                  "tracks_with_reference": int((ref5[:, 0] > 0).sum())}
 
-    out.update(ms_plain=ms_plain, ms_grad_event=ms_grad, ms_grad_event_stored=ms_grad_stored,
-               ms_grad_copies=ms_grad_K, ms_grad_copies_stored=ms_grad_K_stored, its_match=match_out, loopers=loop_out,
+    out.update(ms_plain=ms_plain, ms_grad_event=ms_grad, ms_grad_copies=ms_grad_K, its_match=match_out, loopers=loop_out,
                inefficient=rules_out,
                n_tracks_c5=int(t5.n_tracks.item()), prof=prof,
                weighted_hits=weighted_hits,
@@ -735,11 +732,11 @@ FLOP_FWD, FLOP_ADJ, FLOP_SQRT_FWD = 461, 850, 434
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 
-def stage_flops(u, adjoint_form="checkpoints"):
+def stage_flops(u, form=ADJOINT_FORM):
     """FP32 operations of the Kalman stages: the tracking refit runs the square-root forward step per
-    hit; the gradient runs the forward step, its adjoint and (checkpoint form) the forward step again
-    to recompute the states of each segment."""
-    per_hit = FLOP_FWD + FLOP_ADJ + (FLOP_FWD if adjoint_form == "checkpoints" else 0)
+    hit; the gradient runs the forward step and its adjoint, and in the checkpoint form the forward step
+    again to recompute the states of each segment."""
+    per_hit = FLOP_FWD + FLOP_ADJ + (FLOP_FWD if form == "checkpoints" else 0)
     return {"refit": FLOP_SQRT_FWD * u["n_hits"], "refit_grad": per_hit * u["weighted_hits"]}
 
 
@@ -770,7 +767,8 @@ def finish_native(args, res, world):
     stage_ms = {s: v / k for s, v in prof.items()}
     dom = max(stage_ms, key=lambda s: stage_ms[s])
     byts = stage_bytes(res)
-    n_launch, adj_form = launches_per_step(res["tuning"].get("best"))
+    adj_form = adjoint_form(res)
+    n_launch = LAUNCHES_TRACKING + LAUNCHES_REFIT_GRAD[adj_form]
     flops = stage_flops(res, adj_form)
     fp = res.get("fp32_peak")
     if fp:
@@ -817,16 +815,11 @@ def finish_native(args, res, world):
                     "tracks": res["n_tracks_c5"],
                     "form": "refit + adjoint, the input state of every step stored (80 B per hit; checkpoints "
                             "every 16 steps for tracks of 511 hits and more)",
-                    "stored_states": {"value": res["ms_grad_event_stored"] * 1e3, "unit": "us/event",
-                                      "form": "the same, timed a second time with the shapes that ask for it; "
-                                              "identical gradient"},
                     "batched": {"value": res["ms_grad_copies"] * 1e3 / CENTRAL_COPIES, "unit": "us/event",
                                 "events": CENTRAL_COPIES,
-                                "stored_states": res["ms_grad_copies_stored"] * 1e3 / CENTRAL_COPIES,
                                 "form": "%d copies of the event tracked as one batch, refit + adjoint of all "
-                                        "their tracks in one call (stored_states: timed a second time); "
-                                        "gradient checked to be %d times the event's" % (CENTRAL_COPIES,
-                                                                                          CENTRAL_COPIES)}},
+                                        "their tracks in one call; gradient checked to be %d times the event's" %
+                                        (CENTRAL_COPIES, CENTRAL_COPIES)}},
         "calibration": res["calib"],
         "its_match": res.get("its_match"),
         "looper_legs": res.get("loopers"),
@@ -859,6 +852,10 @@ def finish_native(args, res, world):
         "gpu_launches": n_launch * args.steps,
         "clocks": res["clocks"],
     }
+    if "ms_grad_event_stored" in res:      # a result that timed the stored states beside the checkpoints
+        a = line["adjoint"]
+        a["stored_states"] = {"value": res["ms_grad_event_stored"] * 1e3, "unit": "us/event"}
+        a["batched"]["stored_states"] = res["ms_grad_copies_stored"] * 1e3 / CENTRAL_COPIES
     return line
 
 
@@ -965,12 +962,12 @@ def run_reference(args, rank, world):
 
 # ---------------------------------------------------------------------------------------------
 
-def adjoint_event(form, calls=10):
+def adjoint_event(calls=10):
     """Refit + adjoint of the central calibration event (references from the TPC-ITS matching, raw
-    errors) in one form, library default launch shapes otherwise: ms per call."""
+    errors), library default launch shapes: ms per call."""
     import numpy as np
     import torch
-    from paper_1712_09434_gb300 import capi, tune
+    from paper_1712_09434_gb300 import capi
     dev = "cuda"
     ev = synth.make_event(synth.calib_event())
     cl = capi.Clusters.from_numpy(ev.pad_fp, ev.time_fp, ev.bin_off, 1)
@@ -989,7 +986,6 @@ def adjoint_event(form, calls=10):
     th = torch.tensor(synth.calib_theta(1005), dtype=torch.float64, device=dev)
     s_chi2 = torch.zeros(1, dtype=torch.float64, device=dev)
     grad = torch.zeros(1 + 2 * synth.N_SECTORS, dtype=torch.float64, device=dev)
-    ctx.tpc_set_tuning(tune.to_struct({"refit_grad": (0, 0, 1)}) if form == "stored" else None)
     stream = torch.cuda.current_stream()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ts = []
@@ -1002,7 +998,7 @@ def adjoint_event(form, calls=10):
     st = ctx.tpc_sync_status()
     ctx.close()
     assert st == 0, st
-    return {"adjoint_form": form, "tracks": nt, "ms_per_call": float(np.median(ts)), "calls": calls,
+    return {"adjoint_form": ADJOINT_FORM, "tracks": nt, "ms_per_call": float(np.median(ts)), "calls": calls,
             "note": "--only-adjoint (profiling run)"}
 
 
@@ -1019,9 +1015,9 @@ def main():
     ap.add_argument("--store-tuning", default=None, help="write the autotuned shapes to this JSON cache")
     ap.add_argument("--only-step", action="store_true",
                     help="time the batched step only (no plain/adjoint/e2e/CPU legs); for profiling")
-    ap.add_argument("--only-adjoint", default=None, choices=["checkpoints", "stored"],
-                    help="time the refit + adjoint of the central calibration event only, in one form; "
-                         "for profiling")
+    ap.add_argument("--only-adjoint", default=None, choices=["stored"],
+                    help="time the refit + adjoint of the central calibration event only (stored states, the "
+                         "form the library runs); for profiling")
     ap.add_argument("--fp32-peak", action="store_true",
                     help="measure the FP32 FMA throughput of the GPU only (the roof of the Kalman stages)")
     args = ap.parse_args()
@@ -1035,7 +1031,7 @@ def main():
     if args.only_adjoint:
         import __graft_entry__
         __graft_entry__.build()
-        print(json.dumps(adjoint_event(args.only_adjoint)), flush=True)
+        print(json.dumps(adjoint_event()), flush=True)
         return
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
