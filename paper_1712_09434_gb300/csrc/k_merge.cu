@@ -95,7 +95,6 @@ __global__ void k_merge_fill(Work W) {
         }
         const int b = bin0 + lo;
         const int p = W.mrg_off[b] + atomicSub(W.bin_cnt + b, 1) - 1;
-        W.mrg_list[p] = t;
         merge_firsts(W)[p] = make_int4(e.x, e.y, e.z, t);
     }
 }

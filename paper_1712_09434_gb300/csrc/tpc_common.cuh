@@ -113,7 +113,7 @@ struct Work {
     int32_t *next, *prev;     // [cap_chains]
     int4 *inend;              // [cap_chains] first kept hit (Xtab, Y, Z, sector)
     int32_t *mrg_off;         // [nbins + 1] accepted segments per (event, sector, first row)
-    int32_t *mrg_list;        // [cap_chains] segment indices in mrg_off order
+    int32_t *mrg_list;        // [cap_chains] slice tracks in mrg_off order (slice merge), candidates (looper pairing)
     int4 *outend;             // [cap_chains * 2] (X1, Y1, Z1, sector), (X2, Y2, Z2, row) of the outer end
     int32_t *sec_ymax;        // [max_events * n_sectors] largest |Y| of a segment's first kept hit
     int32_t *head;            // [cap_chains] 1 if the segment starts a merged track
