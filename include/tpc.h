@@ -94,7 +94,10 @@ typedef struct {
 /* Launch shape of the tunable kernels (0 = library default).  Index: 0 grid, 1 links, 2 chains,
  * 3 follow, 4 select, 5 merge, 6 refit, 7 refit_grad.  block = threads per CTA (multiple of 32, at
  * most 256, 128, 256, 128, 1024, 512, 128, 128 by index), ctas_per_sm = CTAs per SM of the grid
- * (<= 64), chunk = work items taken per queue grab (<= 64; used by the following); for the neighbour
+ * (<= 64), chunk = work items taken per queue grab (<= 64; used by the following); a call of up to 2^20
+ * clusters with the plain rules and at most 160 rows follows its few chains in a kernel of fixed shape,
+ * which index 3 does not reach; a ctas_per_sm for the selection (index 4) also makes it take one CTA
+ * per sector, where by default up to four share a sector of a call with few; for the neighbour
  * finding (index 1) chunk = 1 selects the variant that stages rows r+-1 of every bin in shared
  * memory by bulk copies (one CTA per bin) instead of reading them through L1 (a bin's clusters
  * shared by warps, lanes taking them in Z-slab order), and chunk = 2 the L1 variant whose lanes

@@ -9,11 +9,11 @@
 // backwards; tracks too long for the length order keep a checkpoint every CK_K steps instead, from
 // which the reverse pass recomputes each segment's states (same results, bit for bit, with 1772
 // instead of 1311 flop per hit and a local-memory buffer).  Storing took the gradient from 0.38 +
-// 0.82 to 0.35 + 0.43 ms on a central event of 20,000 tracks and from 0.68 + 2.32 to 0.75 + 1.46 ms
-// on 64 events.  The offsets of the warp chunks come out of the length sort.  Per-track chi2 and
-// gradient contributions
-// (s_vd, and (d_k, a_k) for every sector the track visits) are written as records and summed in
-// FP64 in a fixed order (deterministic).
+// 0.82 to 0.35 + 0.43 ms on a central event of 20,000 tracks (0.24 + 0.39 with the items by block
+// index, below) and from 0.68 + 2.32 to 0.75 + 1.46 ms on 64 events.  The offsets of the warp chunks
+// come out of the length sort.  Per-track chi2 and gradient contributions (s_vd, and (d_k, a_k) for
+// every sector the track visits) are written as records and summed in FP64 in a fixed order
+// (deterministic).
 #include "kf.cuh"
 #include "tpc_common.cuh"
 

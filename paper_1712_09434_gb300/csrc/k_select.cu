@@ -285,7 +285,8 @@ void launch_cluster(const Work &W, int items, int block, cudaStream_t s) {
 // of many events 1.  Measured, one / two / four blocks an item: central event 885 / 507 / 320 us (a
 // single block that scans all candidate states every round 1285 us), 5,000-track event 110 / 88 /
 // 74, 5 slices 1005 / 682 / 646 (1460), 12 events 115 / 167 / 229, 64 events 2.14 / 2.52 / 3.39 ms
-// (2.65); groups of 8 were behind 4 everywhere.
+// (2.65); groups of 8 were behind 4 everywhere.  A launch shape with a grid of its own (ctas_per_sm)
+// takes one block an item.
 int group_size(int items, int block, int sm_count) {
     const int slots = sm_count * (1024 / block);
     int cs = 1;
